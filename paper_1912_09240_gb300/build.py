@@ -11,6 +11,8 @@ import os
 import shutil
 import subprocess
 
+from . import normal_tables
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
@@ -29,6 +31,7 @@ def nvcc() -> str:
 
 def _inputs():
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    deps.append(normal_tables.__file__)
     deps.append(os.path.join(ROOT, "include", "pr.h"))
     return deps
 
@@ -47,7 +50,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     cc = nvcc()
     flags = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",
-                    "-I", os.path.join(ROOT, "include")]
+                    "-I", os.path.join(ROOT, "include"), "-I", BUILD]
+    normal_tables.write(os.path.join(BUILD, "normal_tables.h"))
 
     def compile_one(src):
         obj = os.path.join(BUILD, src.replace(".cu", ".o"))

@@ -10,6 +10,7 @@
 // and written once per slice (structure of arrays, coalesced).  The step loop
 // draws its normals from Philox4x32-10 keyed by the seed and counted by
 // (step, particle, slice, problem), so nothing random is stored.
+#include <cuda_pipeline.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -18,8 +19,12 @@
 #include <mutex>
 #include <vector>
 
+#define PR_TABLE_STORAGE static __device__ const __align__(16)
+#include "normal_tables.h"
+
 #include "fine_dev.cuh"
 #include "match.cuh"
+#include "normal64.cuh"
 #include "pr_common.cuh"
 
 namespace pr {
@@ -127,7 +132,7 @@ inline FineSmem fine_smem_layout(int bins, bool any_grid, bool match, bool f32)
 }
 
 struct FineSmemOffsets {
-    unsigned thr, hs, he, match;
+    unsigned thr, hs, he, match, tab;   // tab: the binary64 normals' tables
 };
 
 // ---------------------------------------------------------------------------
@@ -352,11 +357,44 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
 
 // ---------------------------------------------------------------------------
 // binary64 kernel (the plain FP64 path), any fast_dim <= 16, one particle per
-// thread, FP64 normals and arithmetic.
+// thread, binary64 state and arithmetic.
+//
+// Bound by the binary64 pipe (64 cycles of a sub-partition per warp
+// instruction): 8 operations per step of the double well, 6 of the OU family,
+// the pipe 85 % busy.  The normals come from integer arithmetic
+// (normal64.cuh), 232 of the 240 instructions of a step, beside them.  2^17
+// particles x 2 slices x 1000 steps of the double well: 4.71 ms (5.6e10
+// particle-steps/s); 40.8 ms with log, sqrt and sincospi of the CUDA library,
+// which made 80 binary64 operations a step.
+// The normals' tables (92 KB) are copied into the CTA's shared memory where
+// they fit beside the histograms and the matching (SMT), else read through L1.
 // ---------------------------------------------------------------------------
 
+__device__ __forceinline__ void normals_f64(uint32_t w0, uint32_t w1, const NormalTables& tab, double& z0, double& z1)
+{
+    uint64_t b0, b1;
+    box_muller_fixed(w0, w1, tab, b0, b1);
+    z0 = __longlong_as_double((long long)b0);
+    z1 = __longlong_as_double((long long)b1);
+}
+
+// One step of a d = 1 family from its two normals.
 template <int KIND>
-__global__ void __launch_bounds__(128)
+__device__ __forceinline__ void em_step_f64(const FineArgs& a, double& x, double& y, double z0, double z1)
+{
+    if (KIND == PR_MODEL_CHEM) {   // the amplitudes depend on the state
+        em_step_chem_f64(x, y, z0, z1, a.chem_d);
+        return;
+    }
+    const double f = slow_force<KIND == PR_MODEL_OU ? 0 : 1>(x, y, a.lam);
+    const double xn = x - f * a.drift_dt + a.sx * z0;
+    y = y - (y - x) * a.relax + a.sy * z1;
+    x = xn;
+}
+
+// ONE: fast_dim = 1 (state in registers, one Philox block per pair of steps).
+template <int KIND, bool ONE, bool SMT>
+__global__ void __launch_bounds__(512)
 fine_f64_kernel(FineArgs a, FineSmemOffsets so, int flags)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -366,6 +404,13 @@ fine_f64_kernel(FineArgs a, FineSmemOffsets so, int flags)
     const int bins = a.g.bins;
     uint32_t* hist_s = reinterpret_cast<uint32_t*>(smem + so.hs);
     uint32_t* hist_e = reinterpret_cast<uint32_t*>(smem + so.he);
+    if (SMT) {   // in flight while the matching index is built
+        uint4* dst = reinterpret_cast<uint4*>(smem + so.tab);
+        const uint4* src = reinterpret_cast<const uint4*>(kNormalTables);
+        for (int i = threadIdx.x; i < (int)(kNormalTableWords / 2); i += blockDim.x)
+            __pipeline_memcpy_async(dst + i, src + i, 16);
+        __pipeline_commit();
+    }
     MatchSmem ms;
     if (any_grid) {
         for (int i = threadIdx.x; i < bins; i += blockDim.x) {
@@ -377,63 +422,69 @@ fine_f64_kernel(FineArgs a, FineSmemOffsets so, int flags)
             build_match_index(a.g, a.cdf_prior + (size_t)s * (bins + 1),
                               a.cdf_target + (size_t)s * (bins + 1), ms);
         }
-        __syncthreads();
     }
-    const int D = a.fast_dim;
+    if (SMT) __pipeline_wait_prior(0);
+    __syncthreads();
+    const NormalTables tab = normal_tables_at(SMT ? (const void*)(smem + so.tab) : (const void*)kNormalTables);
+    const int D = ONE ? 1 : a.fast_dim;
     const int64_t N = a.n;
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool ok = p < N;
     const double* __restrict__ xin = static_cast<const double*>(a.x_in) + (int64_t)s * a.in_slice_stride;
     const double* __restrict__ yin = static_cast<const double*>(a.y_in) + (int64_t)s * a.in_slice_stride * D;
     double* __restrict__ xout = static_cast<double*>(a.x_out) + (int64_t)s * N;
     double* __restrict__ yout = static_cast<double*>(a.y_out) + (int64_t)s * N * D;
+    const uint32_t k0 = a.k0, k1 = a.k1, chi = a.ctr_hi;
 
-    double x = ok ? xin[p] : 0.0;
-    double y[PR_MAX_FAST_DIM];
-    for (int j = 0; j < D; ++j) y[j] = ok ? yin[(int64_t)j * N + p] : 0.0;
-    if (do_match && ok) x = match_one_f64(ms, a.g, x);
-    if (do_hs && ok) atomicAdd(&hist_s[bin_of_f64(a.g, x)], 1u);
-
-    const uint32_t k0 = a.k0, k1 = a.k1, chi = a.ctr_hi, pid = (uint32_t)p;
-    const int Q = 1 + D;
-    for (int m = 0; m < a.steps; ++m) {
-        double z[PR_MAX_FAST_DIM + 3];
-        if (Q <= 2) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)(m >> 1), pid, slice, chi), k0, k1);
-            if (m & 1) box_muller_f64(w.z, w.w, z[0], z[1]);
-            else box_muller_f64(w.x, w.y, z[0], z[1]);
+    for (int tile = 0; tile < a.tiles_per_cta; ++tile) {
+        const int64_t p = ((int64_t)blockIdx.x * a.tiles_per_cta + tile) * blockDim.x + threadIdx.x;
+        if (p >= N) break;
+        const uint32_t pid = (uint32_t)p;
+        double x = xin[p];
+        double y[ONE ? 1 : PR_MAX_FAST_DIM];
+        for (int j = 0; j < D; ++j) y[j] = yin[(int64_t)j * N + p];
+        if (do_match) x = match_one_f64(ms, a.g, x);
+        if (do_hs) atomicAdd(&hist_s[bin_of_f64(a.g, x)], 1u);
+        if (ONE) {
+            double z0, z1;
+            for (int mp = 0; mp < (a.steps >> 1); ++mp) {
+                const uint4 w = philox4x32_10(make_uint4((uint32_t)mp, pid, slice, chi), k0, k1);
+                normals_f64(w.x, w.y, tab, z0, z1);
+                em_step_f64<KIND>(a, x, y[0], z0, z1);
+                normals_f64(w.z, w.w, tab, z0, z1);
+                em_step_f64<KIND>(a, x, y[0], z0, z1);
+            }
+            if (a.steps & 1) {
+                const uint4 w = philox4x32_10(make_uint4((uint32_t)(a.steps >> 1), pid, slice, chi), k0, k1);
+                normals_f64(w.x, w.y, tab, z0, z1);
+                em_step_f64<KIND>(a, x, y[0], z0, z1);
+            }
         } else {
-            // F full blocks per step, then the step's T = Q mod 4 normals from
-            // the tail blocks shared by its group of four steps
-            const int F = Q / 4, T = Q % 4;
-            for (int gi = 0; gi < F; ++gi) {
-                const uint4 w = philox4x32_10(make_uint4((uint32_t)m, pid, slice, chi | (uint32_t)gi), k0, k1);
-                box_muller_f64(w.x, w.y, z[4 * gi], z[4 * gi + 1]);
-                box_muller_f64(w.z, w.w, z[4 * gi + 2], z[4 * gi + 3]);
-            }
-            for (int i = 0; i < T; ++i) {
-                const int idx = (m & 3) * T + i;
-                const uint4 w = philox4x32_10(make_uint4((uint32_t)(m >> 2), pid, slice, chi | (uint32_t)(F + idx / 4)),
-                                              k0, k1);
-                double za, zb;
-                if ((idx & 2) != 0) box_muller_f64(w.z, w.w, za, zb);
-                else box_muller_f64(w.x, w.y, za, zb);
-                z[4 * F + i] = (idx & 1) ? zb : za;
+            const int Q = 1 + D;
+            for (int m = 0; m < a.steps; ++m) {
+                double z[PR_MAX_FAST_DIM + 3];
+                // F full blocks per step, then the step's T = Q mod 4 normals from
+                // the tail blocks shared by its group of four steps
+                const int F = Q / 4, T = Q % 4;
+                for (int gi = 0; gi < F; ++gi) {
+                    const uint4 w = philox4x32_10(make_uint4((uint32_t)m, pid, slice, chi | (uint32_t)gi), k0, k1);
+                    normals_f64(w.x, w.y, tab, z[4 * gi], z[4 * gi + 1]);
+                    normals_f64(w.z, w.w, tab, z[4 * gi + 2], z[4 * gi + 3]);
+                }
+                for (int i = 0; i < T; ++i) {
+                    const int idx = (m & 3) * T + i;
+                    const uint4 w = philox4x32_10(
+                        make_uint4((uint32_t)(m >> 2), pid, slice, chi | (uint32_t)(F + idx / 4)), k0, k1);
+                    double za, zb;
+                    normals_f64((idx & 2) ? w.z : w.x, (idx & 2) ? w.w : w.y, tab, za, zb);
+                    z[4 * F + i] = (idx & 1) ? zb : za;
+                }
+                double ysum = 0.0;
+                for (int j = 0; j < D; ++j) ysum += y[j];
+                const double f = slow_force<1>(x, ysum / (double)D, a.lam);
+                const double xn = x - f * a.drift_dt + a.sx * z[0];
+                for (int j = 0; j < D; ++j) y[j] = y[j] - (y[j] - x) * a.relax + a.sy * z[1 + j];
+                x = xn;
             }
         }
-        if (KIND == PR_MODEL_CHEM) {   // sx = sy = 1: the amplitudes depend on the state
-            em_step_chem_f64(x, y[0], a.sx * z[0], a.sy * z[1], a.chem_d);
-            continue;
-        }
-        double ysum = 0.0;
-        for (int j = 0; j < D; ++j) ysum += y[j];
-        const double ym = (KIND == PR_MODEL_DW_MULTI) ? ysum / (double)D : y[0];
-        const double f = slow_force<KIND == PR_MODEL_OU ? 0 : 1>(x, ym, a.lam);
-        const double xn = x - f * a.drift_dt + a.sx * z[0];
-        for (int j = 0; j < D; ++j) y[j] = y[j] - (y[j] - x) * a.relax + a.sy * z[1 + j];
-        x = xn;
-    }
-    if (ok) {
         xout[p] = x;
         for (int j = 0; j < D; ++j) yout[(int64_t)j * N + p] = y[j];
         if (do_he) atomicAdd(&hist_e[bin_of_f64(a.g, x)], 1u);
@@ -774,6 +825,36 @@ static pr_status launch_f32_multi(int D, const FineArgs& a, FineSmemOffsets so, 
     }
 }
 
+// Binary64 launch.  CTAs of 512 threads; 256 or 128 where larger ones would
+// leave SMs without a CTA.  Several consecutive tiles per CTA (at most 8,
+// while ~8 waves of CTAs remain) share the prologue.  The tables go to shared
+// memory where they fit and the run is long enough to repay the copy.
+template <int KIND, bool ONE>
+static pr_status launch_f64(const FineArgs& a, FineSmemOffsets so, int flags, size_t smem, int n_slices,
+                            cudaStream_t st)
+{
+    int threads = 512;
+    while (threads > 128 && ((a.n + threads - 1) / threads) * n_slices < 2 * (int64_t)num_sms()) threads >>= 1;
+    FineArgs b = a;
+    const int64_t tiles = (a.n + threads - 1) / threads;
+    const int64_t tpc = tiles * n_slices / ((int64_t)num_sms() * 16);
+    b.tiles_per_cta = (int)std::max<int64_t>(1, std::min<int64_t>(tpc, 8));
+    const dim3 grid((unsigned)((tiles + b.tiles_per_cta - 1) / b.tiles_per_cta), (unsigned)n_slices);
+    const size_t with_tables = align16(smem) + (size_t)kNormalTableWords * 8;
+    if (a.steps >= 16 && with_tables <= (size_t)smem_optin_max()) {
+        so.tab = (unsigned)align16(smem);
+        auto k = fine_f64_kernel<KIND, ONE, true>;
+        PR_TRY_CUDA(set_smem(k, with_tables));
+        k<<<grid, threads, with_tables, st>>>(b, so, flags);
+    } else {
+        auto k = fine_f64_kernel<KIND, ONE, false>;
+        PR_TRY_CUDA(set_smem(k, smem));
+        k<<<grid, threads, smem, st>>>(b, so, flags);
+    }
+    PR_CHECK_LAUNCH();
+    return PR_OK;
+}
+
 static int g_ppt = 0;   // particles per thread of the binary32 d = 1 kernel (0: per launch)
 
 // Particles per thread of a binary32 d = 1 launch over n x n_slices
@@ -877,12 +958,11 @@ extern "C" pr_status pr_fine_propagate(const pr_model* model, pr_precision preci
     a.syk_f = (float)(a.sy * 1.1774100225154746910);
     if (is_chem(model->kind)) {
         // state-dependent amplitudes: dt is folded into the variance
-        // polynomials, so the binary64 normals enter unscaled and the
-        // binary32 ones scaled by sqrt(2 ln 2) alone
+        // polynomials, so the binary64 normals enter unscaled (sx, sy unused)
+        // and the binary32 ones scaled by sqrt(2 ln 2) alone
         const bool printed = model->kind == PR_MODEL_CHEM_PRINTED;
         a.chem_d = make_chem_consts<double>(model->rate, printed, dt, model->tau_x, model->eps);
         a.chem_f = make_chem_consts<float>(model->rate, printed, dt, model->tau_x, model->eps);
-        a.sx = a.sy = 1.0;
         a.sxk_f = a.syk_f = 1.1774100225154746910f;
     }
     a.tiles_per_cta = 1;
@@ -933,7 +1013,7 @@ extern "C" pr_status pr_fine_propagate(const pr_model* model, pr_precision preci
         return pr_fine_propagate(model, precision, rng, x_out, y_out, 0, x_out, y_out, n, slice_begin, n_slices,
                                  steps, dt, grid, nullptr, nullptr, nullptr, nullptr, counts_end, cdf_end, stream);
     }
-    FineSmemOffsets so{(unsigned)L.thr, (unsigned)L.hs, (unsigned)L.he, (unsigned)L.match};
+    FineSmemOffsets so{(unsigned)L.thr, (unsigned)L.hs, (unsigned)L.he, (unsigned)L.match, 0u};
     const int flags = (any_grid ? 1 : 0) | (do_match ? 2 : 0) | (counts_start ? 4 : 0) | (counts_end ? 8 : 0);
     pr_status rc = PR_OK;
     if (precision == PR_F32) {
@@ -963,35 +1043,15 @@ extern "C" pr_status pr_fine_propagate(const pr_model* model, pr_precision preci
             }
         }
     } else {
-        const int threads = 128;
-        dim3 g((unsigned)((n + threads - 1) / threads), (unsigned)n_slices);
         switch (model->kind) {
-        case PR_MODEL_OU: {
-            auto k = fine_f64_kernel<PR_MODEL_OU>;
-            PR_TRY_CUDA(set_smem(k, L.total));
-            k<<<g, threads, L.total, st>>>(a, so, flags);
-            break;
-        }
-        case PR_MODEL_DOUBLE_WELL: {
-            auto k = fine_f64_kernel<PR_MODEL_DOUBLE_WELL>;
-            PR_TRY_CUDA(set_smem(k, L.total));
-            k<<<g, threads, L.total, st>>>(a, so, flags);
-            break;
-        }
+        case PR_MODEL_OU: rc = launch_f64<PR_MODEL_OU, true>(a, so, flags, L.total, n_slices, st); break;
+        case PR_MODEL_DOUBLE_WELL: rc = launch_f64<PR_MODEL_DOUBLE_WELL, true>(a, so, flags, L.total, n_slices, st); break;
         case PR_MODEL_CHEM:
-        case PR_MODEL_CHEM_PRINTED: {
-            auto k = fine_f64_kernel<PR_MODEL_CHEM>;
-            PR_TRY_CUDA(set_smem(k, L.total));
-            k<<<g, threads, L.total, st>>>(a, so, flags);
-            break;
+        case PR_MODEL_CHEM_PRINTED: rc = launch_f64<PR_MODEL_CHEM, true>(a, so, flags, L.total, n_slices, st); break;
+        default:   // (the multi-component family with one component is the double well)
+            rc = D == 1 ? launch_f64<PR_MODEL_DOUBLE_WELL, true>(a, so, flags, L.total, n_slices, st)
+                        : launch_f64<PR_MODEL_DW_MULTI, false>(a, so, flags, L.total, n_slices, st);
         }
-        default: {
-            auto k = fine_f64_kernel<PR_MODEL_DW_MULTI>;
-            PR_TRY_CUDA(set_smem(k, L.total));
-            k<<<g, threads, L.total, st>>>(a, so, flags);
-        }
-        }
-        PR_CHECK_LAUNCH();
     }
     if (rc != PR_OK) return rc;
     if (cdf_start) {

@@ -86,11 +86,6 @@ __device__ __forceinline__ float uniform_f32(uint32_t w)
     return __uint_as_float(0x3F800000u | (w >> 9)) - 0.99999994039535522461f;
 }
 
-__device__ __forceinline__ double uniform_f64(uint32_t w)
-{
-    return ((double)(w >> 9) + 0.5) * (1.0 / 8388608.0);
-}
-
 // Box-Muller in binary32 on the special-function unit: r = sqrt(-2 ln u0),
 // theta = 2 pi u1.  -2 ln u0 = -2 ln2 * log2(u0).
 __device__ __forceinline__ float sqrt_approx(float v)
@@ -212,17 +207,6 @@ inline ChemConsts<T> make_chem_consts(const double* k, bool printed, double dt, 
     c.e2 = (T)((k[2] - 3.0 * k[3]) * ay);
     c.e3 = (T)(k[3] * ay);
     return c;
-}
-
-__device__ __forceinline__ void box_muller_f64(uint32_t w0, uint32_t w1, double& z0, double& z1)
-{
-    const double u0 = uniform_f64(w0);
-    const double u1 = uniform_f64(w1);
-    const double r = sqrt(-2.0 * log(u0));
-    double s, c;
-    sincospi(2.0 * u1, &s, &c);
-    z0 = r * c;
-    z1 = r * s;
 }
 
 // ---------------------------------------------------------------------------
