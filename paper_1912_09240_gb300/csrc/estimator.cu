@@ -3,17 +3,23 @@
 // coordinate v of the ensemble (the slow variable x, or one fast component),
 // q = 1..max_order, with the weights W^p given or uniform (1/n).
 //
-// Each thread accumulates its particles in binary64 registers; a CTA reduces
-// its threads in a fixed tree (warp shuffles, then the warps in order) to one
-// partial per order, and a second kernel adds a slice's partials in block
-// order.  The grid depends only on n and the slice count, so a call returns
-// the same bits every time on any device.  Each order's term enters its sum
-// through one fused multiply-add (W v^(q-1) times v, added with one rounding),
-// and the running power takes one multiply: per particle 2 max_order - 1
-// binary64 operations with weights, 2 max_order - 2 without (the first order
-// adds v itself).  On GB300's narrow FP64 pipe that, not HBM,
-// bounds the pass; it is meant for observables at the end of a run, not for
-// every step.
+// A CTA reduces its threads' binary64 sums in a fixed tree (warp shuffles, then
+// the warps in order) to one partial per order, and a second kernel adds a
+// slice's partials in a fixed order.  The grid depends only on n and the slice
+// count, so a call returns the same bits every time on any device.
+//
+// Binary32 particles without weights (moments_f32_kernel): binary64 arithmetic
+// takes 64 cycles of a sub-partition per warp instruction, so the terms are
+// summed on the binary32 units in four words per order, with every rounding
+// error kept (29 operations per particle for the first two orders); the words
+// enter the binary64 sum once per 128 particles.
+//
+// Weighted sums and binary64 particles (moments_kernel): each order's term
+// enters its sum through one binary64 fused multiply-add (W v^(q-1) times v,
+// added with one rounding), and the running power takes one multiply: per
+// particle 2 max_order - 1 binary64 operations with weights, 2 max_order - 2
+// without (the first order adds v itself).  On GB300's narrow FP64 pipe that,
+// not HBM, bounds the pass.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -27,12 +33,190 @@ constexpr int kMomThreads = 256;
 constexpr int kMomMaxOrder = 4;
 constexpr int kMomUnroll = 8;              // loads in flight per thread
 constexpr int64_t kMomPerBlock = 4096;     // particles per CTA at least (then fewer CTAs)
-constexpr int64_t kMomMaxBlocks = 2432;    // CTAs over all slices at most (16 per SM of 152)
+constexpr int64_t kMomMaxBlocks = 1824;    // CTAs over all slices at most: 12 per SM of 152, two waves of the
+                                           // binary32 kernel's 6 (orders 1, 2), three of its 4 (orders 3, 4)
 
 static int64_t moments_blocks(int64_t n, int32_t n_slices)
 {
     const int64_t cap = std::max<int64_t>(1, kMomMaxBlocks / n_slices);
     return std::min<int64_t>(cap, std::max<int64_t>(1, (n + kMomPerBlock - 1) / kMomPerBlock));
+}
+
+// The CTA's sums of acc, in a fixed order, to its place in `partial`.
+template <int Q>
+__device__ __forceinline__ void reduce_partials(const double (&acc)[Q], double* __restrict__ partial)
+{
+    __shared__ double red[Q][kMomThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        double a = acc[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+        if (lane == 0) red[q][warp] = a;
+    }
+    __syncthreads();
+    if (threadIdx.x < Q) {
+        double t = 0.0;
+        for (int k = 0; k < kMomThreads / 32; ++k) t += red[threadIdx.x][k];
+        partial[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * Q + threadIdx.x] = t;
+    }
+}
+
+// A sum of binary32 terms in four words.  `hi` starts at 1.5 2^k and stays in
+// the binade of 2^k while the terms' sum is below 2^(k-1), so that the rounding
+// error of each addition comes exactly from two more (Dekker 1971, |hi| >= |x|);
+// `mid`, at 1.5 2^(k-15), takes the errors the same way (below 2^(k-24) each),
+// `low`, at 1.5 2^(k-28), those of `mid` (2^(k-39)), and `rest` what is left
+// (2^(k-52)).  For up to kRun terms of at most 2^(k-8), each with up to two
+// terms for add_small.  The sum is kept to about 2^(k-66), the binary64 sum of
+// as many terms to 2^(k-8-53) at best.
+constexpr int kRun = 128;
+
+struct Sum4 {
+    float hi, mid, low, rest;
+
+    __device__ __forceinline__ static float base(int k) { return __int_as_float(((k + 127) << 23) | 0x400000); }
+
+    __device__ __forceinline__ void reset(int k)
+    {
+        hi = base(k);
+        mid = base(k - 15);
+        low = base(k - 28);
+        rest = 0.0f;
+    }
+    // w + x with the error of the addition
+    __device__ __forceinline__ static float into(float& w, float x)
+    {
+        const float s = __fadd_rn(w, x);
+        const float e = __fsub_rn(x, __fsub_rn(s, w));
+        w = s;
+        return e;
+    }
+    __device__ __forceinline__ void add_small(float e) { rest = __fadd_rn(rest, into(low, into(mid, e))); }
+    __device__ __forceinline__ void add(float x) { add_small(into(hi, x)); }
+    __device__ __forceinline__ double value(int k) const
+    {
+        return widen(__fsub_rn(hi, base(k))) + (widen(__fsub_rn(mid, base(k - 15))) +
+                                                (widen(__fsub_rn(low, base(k - 28))) + widen(rest)));
+    }
+};
+
+// the largest of three magnitudes (NaNs are passed over)
+__device__ __forceinline__ float max3_abs(float a, float b, float c)
+{
+    float r;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Exponents e of a bound |v| <= 2^e for which every word and every product's
+// error term of the orders up to Q is a normal binary32 number (or too small
+// to matter: below 2^-57 of one term at the bound).
+template <int Q>
+__device__ __forceinline__ bool run_exponent_ok(int e)
+{
+    return Q * e <= 100 && Q * e >= -40;
+}
+
+// Bound by issue: 40 instructions per particle for the first two orders, 31 of
+// them binary32 additions and products.  49 x 2^20 particles, mean and second
+// moment: 67.6 us with the finishing kernel (211 us with binary64 terms), and
+// closer to the exact sum (1.1e-16 instead of 3.6e-16).
+template <int Q>
+__global__ void __launch_bounds__(kMomThreads, Q <= 2 ? 6 : 4)
+moments_f32_kernel(const float* __restrict__ v, int64_t stride, int64_t n, int64_t per_block,
+                   double* __restrict__ partial)
+{
+    const float* vs = v + (int64_t)blockIdx.y * stride;
+    const int64_t b = (int64_t)blockIdx.x * per_block, e = min(n, b + per_block);
+    double acc[Q];
+    Sum4 sum[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) acc[q] = 0.0;
+    int ex = -1000;          // the run's bound |v| <= 2^ex; -1000: no run open
+    float bound = -1.0f;
+    int taken = 0;
+    auto close_run = [&]() {
+        if (ex > -1000)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) acc[q] += sum[q].value((q + 1) * ex + 8);
+        ex = -1000;
+        bound = -1.0f;
+        taken = 0;
+    };
+    auto open_run = [&](int at) {
+        if (!run_exponent_ok<Q>(at)) return;
+        ex = at;
+        bound = __int_as_float((at + 127) << 23);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) sum[q].reset((q + 1) * ex + 8);
+    };
+    // least e with |v| <= 2^e for the encoding of |v| (not 0)
+    auto exponent_of = [](uint32_t bits) { return (int)(bits >> 23) - 126; };
+    // every thread walks the whole range, so that a warp decides together
+    for (int64_t b0 = b; b0 < e; b0 += kMomUnroll * kMomThreads) {
+        float x[kMomUnroll];
+        float top = 0.0f;
+        if (b0 + kMomUnroll * kMomThreads <= e) {
+            const float* at = vs + b0 + threadIdx.x;
+#pragma unroll
+            for (int k = 0; k < kMomUnroll; ++k) x[k] = __ldcs(at + k * kMomThreads);
+        } else {
+#pragma unroll
+            for (int k = 0; k < kMomUnroll; ++k) {
+                const int64_t p = b0 + (int64_t)k * kMomThreads + threadIdx.x;
+                x[k] = p < e ? vs[p] : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kMomUnroll; k += 2) top = max3_abs(top, x[k], x[k + 1]);
+        if (taken == kRun || __any_sync(0xffffffffu, !(top <= bound))) {
+            // a new run, its bound four times the warp's largest value here, so
+            // that the values to come stay within it
+            close_run();
+            open_run(exponent_of(__reduce_max_sync(0xffffffffu, __float_as_uint(top))) + 2);
+        }
+        if (top <= bound) {   // the whole warp (a NaN takes either way into the sum)
+            taken += kMomUnroll;
+#pragma unroll
+            for (int k = 0; k < kMomUnroll; ++k) {
+                sum[0].add(x[k]);
+                if (Q >= 2) {
+                    // x^2 = p + pe exactly
+                    const float p = __fmul_rn(x[k], x[k]), pe = __fmaf_rn(x[k], x[k], -p);
+                    sum[1].add(p);
+                    sum[1].add_small(pe);
+                    if (Q >= 3) {
+                        const float h = __fmul_rn(p, x[k]);
+                        sum[2].add(h);
+                        sum[2].add_small(__fmaf_rn(p, x[k], -h));
+                        sum[2].add_small(__fmul_rn(pe, x[k]));
+                    }
+                    if (Q >= 4) {
+                        const float h = __fmul_rn(p, p);
+                        sum[3].add(h);
+                        sum[3].add_small(__fmaf_rn(p, p, -h));
+                        sum[3].add_small(__fmul_rn(2.0f * p, pe));
+                    }
+                }
+            }
+        } else {   // values beyond the runs' range: binary64 terms
+#pragma unroll
+            for (int k = 0; k < kMomUnroll; ++k) {
+                const double d = widen(x[k]);
+                double t = d;
+                acc[0] += d;
+#pragma unroll
+                for (int q = 1; q < Q; ++q) {
+                    acc[q] = fma(t, d, acc[q]);
+                    t *= d;
+                }
+            }
+        }
+    }
+    close_run();
+    reduce_partials<Q>(acc, partial);
 }
 
 template <typename T, int Q, bool W>
@@ -79,33 +263,24 @@ moments_kernel(const T* __restrict__ v, int64_t stride, const double* __restrict
             }
         }
     }
-    __shared__ double red[Q][kMomThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        double a = acc[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        if (lane == 0) red[q][warp] = a;
-    }
-    __syncthreads();
-    if (threadIdx.x < Q) {
-        double t = 0.0;
-        for (int k = 0; k < kMomThreads / 32; ++k) t += red[threadIdx.x][k];
-        partial[((int64_t)s * gridDim.x + blockIdx.x) * Q + threadIdx.x] = t;
-    }
+    reduce_partials<Q>(acc, partial);
 }
 
-// out[s][q] = sum of slice s's partials in block order (divided by n without weights)
-__global__ void moments_finish_kernel(const double* __restrict__ partial, int64_t nblk, int32_t n_slices, int Q,
-                                      int64_t n, int weighted, double* __restrict__ out)
+// out[s][q] = sum of slice s's partials (divided by n without weights), one
+// warp per sum: the partials of each lane in block order, then a fixed tree
+__global__ void __launch_bounds__(128)
+moments_finish_kernel(const double* __restrict__ partial, int64_t nblk, int32_t n_slices, int Q, int64_t n,
+                      int weighted, double* __restrict__ out)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (i >= (int64_t)n_slices * Q) return;
+    const int lane = threadIdx.x & 31;
     const int64_t s = i / Q, q = i - s * Q;
     double t = 0.0;
-    for (int64_t b = 0; b < nblk; ++b) t += partial[(s * nblk + b) * Q + q];
-    out[i] = weighted ? t : t / (double)n;
+    for (int64_t b = lane; b < nblk; b += 32) t += partial[(s * nblk + b) * Q + q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) out[i] = weighted ? t : t / (double)n;
 }
 
 template <typename T, int Q>
@@ -116,6 +291,8 @@ static void launch_moments(const void* v, int64_t stride, const double* w, int64
     const dim3 grid((unsigned)nblk, (unsigned)n_slices);
     if (w)
         moments_kernel<T, Q, true><<<grid, kMomThreads, 0, st>>>(static_cast<const T*>(v), stride, w, n, per, partial);
+    else if constexpr (sizeof(T) == 4)
+        moments_f32_kernel<Q><<<grid, kMomThreads, 0, st>>>(static_cast<const float*>(v), stride, n, per, partial);
     else
         moments_kernel<T, Q, false><<<grid, kMomThreads, 0, st>>>(static_cast<const T*>(v), stride, w, n, per, partial);
 }
@@ -163,7 +340,7 @@ extern "C" pr_status pr_moments(pr_precision precision, const void* v, int64_t s
         launch_moments_q<double>(max_order, v, slice_stride, w, n, n_slices, nblk, partial, st);
     PR_CHECK_LAUNCH();
     const int64_t tot = (int64_t)n_slices * max_order;
-    moments_finish_kernel<<<(unsigned)((tot + 127) / 128), 128, 0, st>>>(partial, nblk, n_slices, max_order, n,
+    moments_finish_kernel<<<(unsigned)((tot + 3) / 4), 128, 0, st>>>(partial, nblk, n_slices, max_order, n,
                                                                         w ? 1 : 0, out);
     PR_CHECK_LAUNCH();
     return PR_OK;

@@ -4,6 +4,8 @@ component, with and without weights, binary32 and binary64 ensembles, ragged
 sizes and several slices.  Every term is the same binary64 product on both
 sides; only the order of the additions differs, so the tolerance is a few
 units of rounding of the sum of absolute terms."""
+import math
+
 import numpy as np
 import pytest
 
@@ -152,3 +154,57 @@ def test_moments_many_slices(L, orc):
     v64 = v.double().cpu().numpy()
     got = _gpu_moments(L, L.PR_F32, v, n, torch.tensor(w, device=DEV), n, S, 3)
     _check(got, orc.moments(v64, 3, w), v64, w, 3)
+
+
+def _wide(kind, n):
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal(n)
+    if kind == "scales":      # every magnitude from 2^-60 to 2^20
+        x = x * np.exp2(rng.uniform(-60, 20, n))
+    elif kind == "tiny":      # products below the normal binary32 range
+        x = x * 1e-30
+    elif kind == "huge":      # squares above it
+        x = x * 1e25
+    elif kind == "offset":
+        x = 400.0 + x
+    elif kind == "outlier":
+        x[n // 2] = 3e6
+    elif kind == "growing":   # every run's bound is passed
+        x = x * np.exp2(np.arange(n) * (40.0 / n))
+    elif kind == "zeros":
+        x[:] = 0.0
+        x[::1000] = -0.0
+    return x.astype(np.float32)
+
+
+@pytest.mark.parametrize("kind", ["scales", "tiny", "huge", "offset", "outlier", "growing", "zeros"])
+@pytest.mark.parametrize("n", [5, 2048, 2049, 300001])
+@pytest.mark.parametrize("order", [1, 2, 3, 4])
+def test_binary32_sums_over_the_range_of_values(L, kind, n, order):
+    """The binary32 words hold the sums of any values: within the tolerance of
+    the other tests, 1e-13 of the sum of absolute terms.  The reference is the
+    correctly rounded sum (math.fsum): a running binary64 sum of 3e5 terms is
+    itself off by up to 1e-13."""
+    x = _wide(kind, n)
+    ws = torch.empty(L.pr_moments_workspace(n, 1, order), dtype=torch.uint8, device=DEV)
+    out = torch.empty(1, order, dtype=torch.float64, device=DEV)
+    L.pr_moments(L.PR_F32, torch.from_numpy(x).to(DEV), n, None, n, 1, order, out, ws)
+    got = out.cpu().numpy()[0]
+    ref = np.array([math.fsum(x.astype(np.float64) ** (q + 1)) / n for q in range(order)])
+    scale = np.array([np.mean(np.abs(x.astype(np.float64)) ** (q + 1)) for q in range(order)])
+    assert np.all(np.abs(got - ref) <= 1e-13 * scale)
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("where", [0, 7, 2047, 40000])
+def test_non_finite_values(L, bad, where):
+    n = 50000
+    x = np.random.default_rng(1).standard_normal(n).astype(np.float32)
+    x[where] = bad
+    for order in (1, 2, 4):
+        ws = torch.empty(L.pr_moments_workspace(n, 1, order), dtype=torch.uint8, device=DEV)
+        out = torch.empty(1, order, dtype=torch.float64, device=DEV)
+        L.pr_moments(L.PR_F32, torch.from_numpy(x).to(DEV), n, None, n, 1, order, out, ws)
+        with np.errstate(invalid="ignore"):
+            want = [np.sum(x.astype(np.float64) ** (q + 1)) for q in range(order)]
+        np.testing.assert_array_equal(out.cpu().numpy()[0], want)
