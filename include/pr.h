@@ -515,7 +515,7 @@ pr_status pr_order_statistics(const float* x, int64_t n, const int64_t* ranks, i
  * One iteration = a persistent fine kernel whose CTAs take work items
  * (problem, slice, particle range of about `item_work` particle-steps) from
  * an atomic counter, largest first; counts -> CDFs; the coarse step on every
- * start state; the serial update, one CTA per problem.  From the second
+ * start state; the serial update, one cluster of CTAs per problem.  From the second
  * iteration on it is replayed as a CUDA graph.  Calls on one plan must not
  * overlap.
  */

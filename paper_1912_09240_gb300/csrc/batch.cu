@@ -8,7 +8,7 @@
 //      pr_fine_propagate (fine_dev.cuh), bit for bit;
 //   2. counts -> CDFs for every (problem, slice);
 //   3. the coarse step on every start state (each problem its own P);
-//   4. the serial update of Section 3.2.3, one CTA per problem.
+//   4. the serial update of Section 3.2.3, one cluster of CTAs per problem.
 // From the second iteration on, an iteration is replayed as a CUDA graph
 // (one per parity of the ping-pong buffers).  Items are sized by an amount of
 // work (particle-steps) so that problems with 10^4x different costs balance;
@@ -204,15 +204,18 @@ batch_coarse_kernel(const BatchProblemDev* __restrict__ probs, const BatchRowDev
     for (int i = threadIdx.x; i <= I; i += blockDim.x) dst[i] = out[i];
 }
 
-__global__ void __launch_bounds__(kCoarseThreads)
+// The serial update of one problem on a cluster of CL CTAs (the bits do not depend on CL).
+template <int CL>
+__global__ void __launch_bounds__(kCoarseThreads, 1)
 batch_update_kernel(const BatchProblemDev* __restrict__ probs, int iterator, int qmode,
                     const double* __restrict__ cdf0, const double* __restrict__ fstar,
                     const double* __restrict__ cstar, double* __restrict__ rho, int32_t* __restrict__ status)
 {
     extern __shared__ __align__(16) unsigned char usm[];
-    const BatchProblemDev& P = probs[blockIdx.x];
-    serial_sweep(usm, P.P, P.g, iterator, qmode, P.K, cdf0 + P.c0_off, fstar ? fstar + P.c_off : nullptr,
-                 cstar ? cstar + P.c_off : nullptr, rho + P.r_off, status + blockIdx.x);
+    const int p = blockIdx.x / CL;
+    const BatchProblemDev& P = probs[p];
+    serial_sweep<CL>(usm, P.P, P.g, iterator, qmode, P.K, cdf0 + P.c0_off, fstar ? fstar + P.c_off : nullptr,
+                     cstar ? cstar + P.c_off : nullptr, rho + P.r_off, status + p);
 }
 
 __global__ void batch_restrict0_kernel(const BatchProblemDev* __restrict__ probs, const float* __restrict__ x0,
@@ -268,7 +271,7 @@ struct BatchPlan {
     std::vector<void*> coarse;
     std::vector<BatchProblemDev> hp;
     std::vector<BatchRowDev> hrows;
-    int max_bins = 1;
+    int max_bins = 1, min_bins = PR_MAX_BINS;
     int64_t sumN = 0, sumKN = 0, sumKI = 0, sumKI1 = 0, sumK1I1 = 0, sumI1 = 0, sumK = 0;
     int64_t work = 0;   // particle-steps per iteration
     // device
@@ -395,6 +398,48 @@ static pr_status launch_fine(BatchPlan& pl, int first, int steps_div, cudaStream
     return PR_OK;
 }
 
+// Serial updates of all problems, each on the largest cluster that gives every
+// problem SMs of its own (one CTA per SM: the sweep is a serial chain whose
+// binary64 work the cluster splits); grids below 64 bins take one CTA, as in
+// pr_parareal_update.  16 problems x 32 slices of 256 bins: the coarse sweep
+// 1.17 ms on one CTA each and 0.45 ms on eight, the quantile sweep 2.8 and 1.7 ms.
+static pr_status launch_update(BatchPlan& pl, int iterator, const double* fstar, const double* cstar, cudaStream_t st)
+{
+    int cl = 1;
+    if (pl.min_bins >= 64)
+        for (int c : {8, 4, 2})
+            if ((int64_t)pl.np * c <= num_sms()) {
+                cl = c;
+                break;
+            }
+    auto launch = [&](auto kernel) -> cudaError_t {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(pl.np * cl));
+        cfg.blockDim = dim3(kCoarseThreads);
+        cfg.dynamicSmemBytes = update_smem(pl.max_bins);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)cl;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = cl > 1 ? 1 : 0;
+        return cudaLaunchKernelEx(&cfg, kernel, (const BatchProblemDev*)pl.d_probs, iterator, (int)pl.qmode,
+                                  (const double*)pl.cdf0, fstar, cstar, pl.rho, pl.status);
+    };
+    cudaError_t e;
+    switch (cl) {
+    case 8: e = launch(batch_update_kernel<8>); break;
+    case 4: e = launch(batch_update_kernel<4>); break;
+    case 2: e = launch(batch_update_kernel<2>); break;
+    default: e = launch(batch_update_kernel<1>);
+    }
+    if (e != cudaSuccess) return PR_ERR_CUDA;
+    PR_CHECK_LAUNCH();
+    return PR_OK;
+}
+
 static pr_status enqueue_iteration(BatchPlan& pl, int first, cudaStream_t st)
 {
     pr_status rc = launch_fine(pl, first, 1, st);
@@ -402,13 +447,9 @@ static pr_status enqueue_iteration(BatchPlan& pl, int first, cudaStream_t st)
     batch_cdf_kernel<<<dim3((unsigned)pl.sumK, 2), 256, 0, st>>>(pl.d_probs, pl.d_rows, pl.counts,
                                                                  pl.counts + pl.sumKI, pl.start, pl.fstar);
     PR_CHECK_LAUNCH();
-    const size_t csm = ((size_t)2 * (pl.max_bins + 1) + 2 * (size_t)pl.max_bins + 40) * sizeof(double);
-    batch_coarse_kernel<<<(unsigned)pl.sumK, kCoarseThreads, csm, st>>>(pl.d_probs, pl.d_rows, pl.start, pl.cstar);
+    batch_coarse_kernel<<<(unsigned)pl.sumK, kCoarseThreads, coarse_apply_smem(pl.max_bins), st>>>(pl.d_probs, pl.d_rows, pl.start, pl.cstar);
     PR_CHECK_LAUNCH();
-    batch_update_kernel<<<pl.np, kCoarseThreads, update_smem(pl.max_bins), st>>>(
-        pl.d_probs, (int)pl.iterator, (int)pl.qmode, pl.cdf0, pl.fstar, pl.cstar, pl.rho, pl.status);
-    PR_CHECK_LAUNCH();
-    return PR_OK;
+    return launch_update(pl, (int)pl.iterator, pl.fstar, pl.cstar, st);
 }
 
 static void swap_buffers(BatchPlan& pl)
@@ -505,6 +546,7 @@ extern "C" pr_status pr_batch_create(const pr_problem* problems, int32_t n_probl
         pl->sumI1 += q.grid.bins + 1;
         pl->sumK += q.n_slices;
         pl->max_bins = std::max(pl->max_bins, q.grid.bins);
+        pl->min_bins = std::min(pl->min_bins, q.grid.bins);
         pl->work += q.n * (int64_t)q.n_slices * q.steps;
         for (int s = 0; s < q.n_slices; ++s) pl->hrows.push_back(BatchRowDev{p, s});
         void* h = nullptr;
@@ -568,10 +610,15 @@ extern "C" pr_status pr_batch_create(const pr_problem* problems, int32_t n_probl
     cudaFuncSetAttribute(batch_fine_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
     cudaFuncSetAttribute(batch_fine_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
     cudaFuncSetAttribute(batch_fine_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
-    cudaFuncSetAttribute(batch_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)update_smem(pl->max_bins));
+    auto allow_update = [&](auto kernel) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)update_smem(pl->max_bins));
+    };
+    allow_update(batch_update_kernel<1>);
+    allow_update(batch_update_kernel<2>);
+    allow_update(batch_update_kernel<4>);
+    allow_update(batch_update_kernel<8>);
     cudaFuncSetAttribute(batch_coarse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(((size_t)2 * (pl->max_bins + 1) + 2 * (size_t)pl->max_bins + 40) * sizeof(double)));
+                         (int)coarse_apply_smem(pl->max_bins));
     cudaFuncSetAttribute(batch_restrict0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)((((size_t)(pl->max_bins + 1) * 4 + 15) & ~(size_t)15) + (size_t)pl->max_bins * 4));
     pl->ppt = 4;
@@ -618,9 +665,8 @@ extern "C" pr_status pr_batch_set_initial(void* plan, const float* x0, const flo
     batch_restrict0_kernel<<<pl->np, 256, rsm, st>>>(pl->d_probs, pl->x0, pl->counts0, pl->cdf0);
     PR_CHECK_LAUNCH();
     // zeroth iteration: serial coarse sweep from R X_0
-    batch_update_kernel<<<pl->np, kCoarseThreads, update_smem(pl->max_bins), st>>>(
-        pl->d_probs, (int)PR_ITER_NONE, (int)pl->qmode, pl->cdf0, nullptr, nullptr, pl->rho, pl->status);
-    PR_CHECK_LAUNCH();
+    const pr_status rc = launch_update(*pl, (int)PR_ITER_NONE, nullptr, nullptr, st);
+    if (rc != PR_OK) return rc;
     pl->k = 0;
     return PR_OK;
 }

@@ -302,7 +302,7 @@ coarse_fp_kernel(const double* __restrict__ P, int I, const double* __restrict__
 // The serial sweep of Section 3.2.3 on one CTA (CL = 1) or on a cluster of
 // CL CTAs (launched with that cluster size).
 template <int CL>
-__global__ void __launch_bounds__(kCoarseThreads)
+__global__ void __launch_bounds__(kCoarseThreads, 1)
 parareal_update_kernel(const double* __restrict__ P, GridDev g, int iterator, int qmode, int K,
                        const double* __restrict__ cdf0, const double* __restrict__ fstar,
                        const double* __restrict__ cstar, double* __restrict__ next, int32_t* status)
@@ -311,7 +311,7 @@ parareal_update_kernel(const double* __restrict__ P, GridDev g, int iterator, in
     serial_sweep<CL>(usm, P, g, iterator, qmode, K, cdf0, fstar, cstar, next, status);
 }
 
-__global__ void __launch_bounds__(kCoarseThreads)
+__global__ void __launch_bounds__(kCoarseThreads, 1)
 iterate_kernel(GridDev g, int iterator, int qmode, const double* __restrict__ a, const double* __restrict__ b,
                const double* __restrict__ c, double* __restrict__ out, int32_t* status)
 {
@@ -323,6 +323,7 @@ iterate_kernel(GridDev g, int iterator, int qmode, const double* __restrict__ a,
     double* Ob = Cb + (I + 1);
     JqSmem js = carve_jq(reinterpret_cast<unsigned char*>(Ob + (I + 1)), I);
     if (threadIdx.x == 0) js.flag[1] = 0;
+    fill_edges(g, js);
     const size_t off = (size_t)blockIdx.x * (I + 1);
     for (int i = threadIdx.x; i <= I; i += blockDim.x) {
         Ab[i] = a[off + i];
