@@ -74,15 +74,18 @@ struct BatchFineArgs {
     int steps_div;   // > 1: every item runs ceil(steps / steps_div) steps (timing trials only)
 };
 
+// after thresholds, histograms and matching: the shared Philox rounds of the CTA's warps
+constexpr size_t kBatchRounds = (size_t)(kD1Threads / 32) * 512;
+
 __host__ __device__ inline size_t batch_fine_smem(int max_bins)
 {
     const size_t a = ((size_t)(max_bins + 1) * 4 + 15) & ~(size_t)15;
     const size_t b = ((size_t)max_bins * 4 + 15) & ~(size_t)15;
-    return a + 2 * b + match_smem_bytes_f32(max_bins);
+    return a + 2 * b + match_smem_bytes_f32(max_bins) + kBatchRounds;
 }
 
 template <int PPT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kD1Threads, PPT == 1 ? 6 : PPT == 2 ? 4 : 3)
 batch_fine_kernel(BatchFineArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -94,6 +97,7 @@ batch_fine_kernel(BatchFineArgs a)
     uint32_t* hs = reinterpret_cast<uint32_t*>(smem + off_h);
     uint32_t* he = reinterpret_cast<uint32_t*>(smem + off_h + hb);
     unsigned char* mbase = smem + off_h + 2 * hb;
+    uint4* rounds = reinterpret_cast<uint4*>(mbase + match_smem_bytes_f32(MB));
     for (;;) {
         if (threadIdx.x == 0) s_item = (int)atomicAdd(a.counter, 1u);
         __syncthreads();
@@ -130,7 +134,7 @@ batch_fine_kernel(BatchFineArgs a)
         float* yout = a.yb + P.x_off + (int64_t)s * n;
         const int steps = a.steps_div > 1 ? (P.steps + a.steps_div - 1) / a.steps_div : P.steps;
         const D1Consts c{P.lam, P.ddt, P.rel, P.sxk, P.syk, P.k0, P.k1, P.chi};
-        const D1Smem sm{thr, hs, he, &ms, bf, do_match, true, true};
+        const D1Smem sm{thr, hs, he, &ms, bf, do_match, true, true, rounds};
         if (P.kind == PR_MODEL_OU)
             fine_d1_range<PR_MODEL_OU, PPT>(xin, yin, xout, yout, it.begin, it.end, (uint32_t)s, steps, c, sm);
         else
@@ -621,7 +625,7 @@ extern "C" pr_status pr_batch_create(const pr_problem* problems, int32_t n_probl
                          (int)coarse_apply_smem(pl->max_bins));
     cudaFuncSetAttribute(batch_restrict0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)((((size_t)(pl->max_bins + 1) * 4 + 15) & ~(size_t)15) + (size_t)pl->max_bins * 4));
-    pl->ppt = 4;
+    pl->ppt = 2;   // 16 problems of 1e4..1e5 particles: an iteration 21.8 ms (four particles per thread 22.1 ms)
     pl->item_work = 0.0;
     {
         const int slots = resident_ctas(*pl);

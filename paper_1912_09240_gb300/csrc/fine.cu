@@ -95,31 +95,36 @@ struct FineArgs {
 };
 
 // Dynamic shared memory of the fine kernels: [thresholds | hist_start |
-// hist_end | match table], each section 16-byte aligned.
+// hist_end | match table | shared Philox rounds], each section 16-byte aligned.
 struct FineSmem {
-    size_t thr, hs, he, match, total;
+    size_t thr, hs, he, match, rounds, total;
 };
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
 
 // Binary32 with matching: thresholds, the matching table, then its build
-// scratch, which the two histograms reuse once the table is built.  Binary64
-// (or no matching): thresholds, histograms, then the full matching scratch.
-inline FineSmem fine_smem_layout(int bins, bool any_grid, bool match, bool f32)
+// scratch, which the two histograms and the shared Philox rounds of the CTA's
+// warps (512 bytes each) reuse once the table is built: large grids need no
+// more shared memory for them.  Binary64 (or no matching): thresholds,
+// histograms, then the full matching scratch (binary64) or the rounds.
+inline FineSmem fine_smem_layout(int bins, bool any_grid, bool match, bool f32, int threads)
 {
-    FineSmem L{0, 0, 0, 0, 0};
-    if (!any_grid) return L;
+    FineSmem L{0, 0, 0, 0, 0, 0};
+    const size_t rounds = f32 ? (size_t)(threads / 32) * 512 : 0;
     size_t off = 0;
-    L.thr = off;
-    off += align16((size_t)(bins + 1) * sizeof(float));
-    const size_t hb = align16((size_t)bins * sizeof(uint32_t));
-    if (match && f32) {
-        L.match = off;
-        off += match_table_bytes(bins);
-        L.hs = off;
-        L.he = off + hb;
-        off += std::max(match_build_bytes_f32(bins), 2 * hb);
-    } else {
+    if (any_grid) {
+        L.thr = off;
+        off += align16((size_t)(bins + 1) * sizeof(float));
+        const size_t hb = align16((size_t)bins * sizeof(uint32_t));
+        if (match && f32) {
+            L.match = off;
+            off += match_table_bytes(bins);
+            L.hs = off;
+            L.he = off + hb;
+            L.rounds = off + 2 * hb;
+            L.total = std::max(off + match_build_bytes_f32(bins), L.rounds + rounds);
+            return L;
+        }
         L.hs = off;
         off += hb;
         L.he = off;
@@ -127,12 +132,14 @@ inline FineSmem fine_smem_layout(int bins, bool any_grid, bool match, bool f32)
         L.match = off;
         if (match) off += match_smem_bytes(bins);
     }
-    L.total = off;
+    L.rounds = off;
+    L.total = off + rounds;
     return L;
 }
 
 struct FineSmemOffsets {
-    unsigned thr, hs, he, match, tab;   // tab: the binary64 normals' tables
+    unsigned thr, hs, he, match, rounds;
+    unsigned tab;   // the binary64 normals' tables
 };
 
 // ---------------------------------------------------------------------------
@@ -150,8 +157,11 @@ __device__ __forceinline__ T slow_force(T x, T ymean, T lam)
 // binary32 kernel, fast_dim = 1
 // ---------------------------------------------------------------------------
 
+// CTAs per SM that the registers are cut for: three at four particles per
+// thread (the double-well iteration 72.8 ms; 75.4 with four CTAs and 64
+// registers, 74.7 with five and 48), four at two, eight at one.
 template <int KIND, int PPT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kD1Threads, PPT == 1 ? 8 : PPT == 2 ? 4 : 3)
 fine_f32_d1_kernel(FineArgs a, FineSmemOffsets so, int flags)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -184,7 +194,7 @@ fine_f32_d1_kernel(FineArgs a, FineSmemOffsets so, int flags)
     float* __restrict__ xout = static_cast<float*>(a.x_out) + (int64_t)s * N;
     float* __restrict__ yout = static_cast<float*>(a.y_out) + (int64_t)s * N;
     D1Consts cst{a.lam_f, a.drift_dt_f, a.relax_f, a.sxk_f, a.syk_f, a.k0, a.k1, a.ctr_hi, a.chem_f};
-    D1Smem sm{thr, hist_s, hist_e, &ms, bf, do_match, do_hs, do_he};
+    D1Smem sm{thr, hist_s, hist_e, &ms, bf, do_match, do_hs, do_he, reinterpret_cast<uint4*>(smem + so.rounds)};
     const int64_t span = (int64_t)a.tiles_per_cta * blockDim.x * PPT;
     const int64_t p_begin = (int64_t)blockIdx.x * span;
     fine_d1_range<KIND, PPT>(xin, yin, xout, yout, p_begin, min(N, p_begin + span), slice, a.steps, cst, sm);
@@ -258,6 +268,22 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
     constexpr int FP = F > 0 ? 2 * F : 1;   // Box-Muller pairs of the full blocks
     constexpr int TP = T > 0 ? 2 * T : 1;   // pairs of a group's tail blocks
     const uint32_t k0 = a.k0, k1 = a.k1, chi = a.ctr_hi, pid = (uint32_t)p;
+    // The rounds' part that all particles share, for kSpan steps at a time: a
+    // lane makes block g of step m, the warp reads it back from shared memory.
+    constexpr int kSpan = F > 0 ? (F == 1 ? 32 : F == 2 ? 16 : 8) : 4;   // a multiple of 4, F kSpan <= 32
+    uint4* shared_rounds = reinterpret_cast<uint4*>(smem + so.rounds) + 32 * (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    const PhiloxParticle own = philox_particle(pid, slice, k0);
+    auto fill_rounds = [&](int m) {
+        if (F > 0) {
+            __syncwarp();
+            if (lane < F * kSpan)
+                shared_rounds[lane] =
+                    philox_shared((uint32_t)(m + lane / (F > 0 ? F : 1)), slice, chi | (uint32_t)(lane % (F > 0 ? F : 1)),
+                                  k0, k1);
+            __syncwarp();
+        }
+    };
     // normal 2i of a pair is sqrt(2 ln 2) q_i cos(theta_i), normal 2i + 1 the
     // sine; sqrt(2 ln 2) is folded into the amplitudes sxk, syk
     float tq[TP], tc[TP], ts[TP], tamp[TP];
@@ -265,7 +291,7 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
     auto tail_blocks = [&](int m) {
 #pragma unroll
         for (int j = 0; j < T; ++j) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)(m >> 2), pid, slice, chi | (uint32_t)(F + j)),
+            const uint4 w = philox_finish(own, philox_shared((uint32_t)(m >> 2), slice, chi | (uint32_t)(F + j), k0, k1),
                                           k0, k1);
             box_muller_qcs(w.x, w.y, tq[2 * j], tc[2 * j], ts[2 * j]);
             box_muller_qcs(w.z, w.w, tq[2 * j + 1], tc[2 * j + 1], ts[2 * j + 1]);
@@ -277,14 +303,14 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
     auto step = [&](int m, int s4) {
         float pq = 0.0f, pc = 0.0f, ps = 0.0f;   // Q = 2: this step's pair
         if (Q <= 2) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)(m >> 1), pid, slice, chi), k0, k1);
+            const uint4 w = philox_finish(own, philox_shared((uint32_t)(m >> 1), slice, chi, k0, k1), k0, k1);
             if (m & 1) box_muller_qcs(w.z, w.w, pq, pc, ps);
             else box_muller_qcs(w.x, w.y, pq, pc, ps);
         }
         float q[FP], c[FP], sn[FP], amp[FP];
 #pragma unroll
         for (int gi = 0; gi < F; ++gi) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)m, pid, slice, chi | (uint32_t)gi), k0, k1);
+            const uint4 w = philox_finish(own, shared_rounds[(m % kSpan) * F + gi], k0, k1);
             box_muller_qcs(w.x, w.y, q[2 * gi], c[2 * gi], sn[2 * gi]);
             box_muller_qcs(w.z, w.w, q[2 * gi + 1], c[2 * gi + 1], sn[2 * gi + 1]);
         }
@@ -333,13 +359,17 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
     int m0 = 0;
     if (T > 0) {
         for (; m0 + 4 <= a.steps; m0 += 4) {
+            if (m0 % kSpan == 0) fill_rounds(m0);
             tail_blocks(m0);
 #pragma unroll
             for (int s4 = 0; s4 < 4; ++s4) step(m0 + s4, s4);
         }
         if (m0 < a.steps) tail_blocks(m0);
     }
-    for (int m = m0; m < a.steps; ++m) step(m, m & 3);
+    for (int m = m0; m < a.steps; ++m) {
+        if (m % kSpan == 0) fill_rounds(m);
+        step(m, m & 3);
+    }
     if (ok) {
         xout[p] = x;
 #pragma unroll
@@ -774,11 +804,20 @@ static cudaError_t set_smem(K kernel, size_t bytes)
 
 static int g_tiles_max = 8;   // upper bound of tiles per CTA (binary32 d = 1 kernel)
 
+// Threads per CTA of the binary32 kernels.  The multi-component kernel takes
+// 512: the matching table (up to ~90 KB at 1024 bins) allows two CTAs per SM, so
+// larger CTAs keep more warps resident.
+static int fine_f32_threads(int64_t n, bool multi)
+{
+    if (multi) return n >= 16384 ? 512 : (n >= 4096 ? 256 : 64);
+    return n >= 4096 ? kD1Threads : 64;
+}
+
 template <int KIND, int PPT>
 static pr_status launch_f32_d1(const FineArgs& a, FineSmemOffsets so, int flags, size_t smem,
                                int n_slices, cudaStream_t st)
 {
-    const int threads = a.n >= 4096 ? 256 : 64;
+    const int threads = fine_f32_threads(a.n, false);
     const int64_t per = (int64_t)threads * PPT;
     const int64_t tiles = (a.n + per - 1) / per;
     // Several consecutive tiles per CTA amortise the per-CTA prologue (edge
@@ -800,9 +839,7 @@ template <int KIND, int D>
 static pr_status launch_f32_dn(const FineArgs& a, FineSmemOffsets so, int flags, size_t smem,
                                int n_slices, cudaStream_t st)
 {
-    // 512 threads: the matching table (up to ~90 KB at 1024 bins) allows two
-    // CTAs per SM, so larger CTAs keep more warps resident
-    const int threads = a.n >= 16384 ? 512 : (a.n >= 4096 ? 256 : 64);
+    const int threads = fine_f32_threads(a.n, true);
     dim3 grid((unsigned)((a.n + threads - 1) / threads), (unsigned)n_slices);
     auto k = fine_f32_dn_kernel<KIND, D>;
     PR_TRY_CUDA(set_smem(k, smem));
@@ -984,7 +1021,8 @@ extern "C" pr_status pr_fine_propagate(const pr_model* model, pr_precision preci
     if (counts_start) PR_TRY_CUDA(cudaMemsetAsync(counts_start, 0, (size_t)n_slices * bins * 4, st));
     if (counts_end) PR_TRY_CUDA(cudaMemsetAsync(counts_end, 0, (size_t)n_slices * bins * 4, st));
 
-    const FineSmem L = fine_smem_layout(bins, any_grid, do_match, precision == PR_F32);
+    const int threads = fine_f32_threads(n, D > 1);   // (of the binary32 kernels)
+    const FineSmem L = fine_smem_layout(bins, any_grid, do_match, precision == PR_F32, threads);
     if (L.total > (size_t)smem_optin_max()) {
         if (precision != PR_F32 || !do_match) return PR_ERR_UNSUPPORTED;
         // Binary32 on a grid whose matching table does not fit beside the
@@ -1013,7 +1051,7 @@ extern "C" pr_status pr_fine_propagate(const pr_model* model, pr_precision preci
         return pr_fine_propagate(model, precision, rng, x_out, y_out, 0, x_out, y_out, n, slice_begin, n_slices,
                                  steps, dt, grid, nullptr, nullptr, nullptr, nullptr, counts_end, cdf_end, stream);
     }
-    FineSmemOffsets so{(unsigned)L.thr, (unsigned)L.hs, (unsigned)L.he, (unsigned)L.match, 0u};
+    FineSmemOffsets so{(unsigned)L.thr, (unsigned)L.hs, (unsigned)L.he, (unsigned)L.match, (unsigned)L.rounds, 0u};
     const int flags = (any_grid ? 1 : 0) | (do_match ? 2 : 0) | (counts_start ? 4 : 0) | (counts_end ? 8 : 0);
     pr_status rc = PR_OK;
     if (precision == PR_F32) {

@@ -78,6 +78,47 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
     return c;
 }
 
+// Philox4x32-10 of the counter (c, p, slice, hi) in two parts, for kernels whose
+// lanes differ in the particle p only: what the first three rounds make of
+// (c, slice, hi), the same for every lane, and of (p, slice), the same for every
+// c.  Of the 20 products 15 are left per block, and 17 of the xors.
+struct PhiloxParticle {
+    uint32_t h, l;   // second round's product of the particle's word
+};
+
+__device__ __forceinline__ PhiloxParticle philox_particle(uint32_t p, uint32_t slice, uint32_t k0)
+{
+    const uint32_t x1 = __umulhi(kPhiloxMulB, slice) ^ p ^ k0;
+    const unsigned long long pa = (unsigned long long)kPhiloxMulA * x1;
+    return PhiloxParticle{(uint32_t)(pa >> 32), (uint32_t)pa};
+}
+
+__device__ __forceinline__ uint4 philox_shared(uint32_t c, uint32_t slice, uint32_t hi, uint32_t k0, uint32_t k1)
+{
+    const unsigned long long pa1 = (unsigned long long)kPhiloxMulA * c;
+    const uint32_t z1 = (uint32_t)(pa1 >> 32) ^ hi ^ k1;
+    const unsigned long long pb2 = (unsigned long long)kPhiloxMulB * z1;
+    const uint32_t x2 = (uint32_t)(pb2 >> 32) ^ (kPhiloxMulB * slice) ^ (k0 + kPhiloxWeylA);
+    const unsigned long long pa3 = (unsigned long long)kPhiloxMulA * x2;
+    return make_uint4((uint32_t)pa1 ^ (k1 + kPhiloxWeylB), (uint32_t)pb2 ^ (k0 + 2u * kPhiloxWeylA),
+                      (uint32_t)(pa3 >> 32) ^ (k1 + 2u * kPhiloxWeylB), (uint32_t)pa3);
+}
+
+__device__ __forceinline__ uint4 philox_finish(const PhiloxParticle& p, const uint4& sh, uint32_t k0, uint32_t k1)
+{
+    const unsigned long long pb3 = (unsigned long long)kPhiloxMulB * (p.h ^ sh.x);
+    uint4 v = make_uint4((uint32_t)(pb3 >> 32) ^ sh.y, (uint32_t)pb3, sh.z ^ p.l, sh.w);
+    k0 += 3u * kPhiloxWeylA;
+    k1 += 3u * kPhiloxWeylB;
+#pragma unroll
+    for (int r = 3; r < 10; ++r) {
+        v = philox_round(v, k0, k1);
+        k0 += kPhiloxWeylA;
+        k1 += kPhiloxWeylB;
+    }
+    return v;
+}
+
 // Uniform in (0,1): the odd 24-bit integer 2*(w >> 9) + 1 times 2^-24.
 // In binary32 this is built from the exponent bits of 1.0: the float
 // 1 + (w>>9) 2^-23 minus (1 - 2^-24), an exact subtraction (Sterbenz).
@@ -86,8 +127,6 @@ __device__ __forceinline__ float uniform_f32(uint32_t w)
     return __uint_as_float(0x3F800000u | (w >> 9)) - 0.99999994039535522461f;
 }
 
-// Box-Muller in binary32 on the special-function unit: r = sqrt(-2 ln u0),
-// theta = 2 pi u1.  -2 ln u0 = -2 ln2 * log2(u0).
 __device__ __forceinline__ float sqrt_approx(float v)
 {
     float r;
@@ -95,19 +134,18 @@ __device__ __forceinline__ float sqrt_approx(float v)
     return r;
 }
 
-__device__ __forceinline__ void box_muller_f32(uint32_t w0, uint32_t w1, float& z0, float& z1)
+// log2 of a normal number (a uniform is at least 2^-24): without the scaling
+// that lg2.approx takes for subnormal arguments, four of 60 issue cycles of an
+// Euler-Maruyama step.
+__device__ __forceinline__ float log2_normal(float v)
 {
-    const float u0 = uniform_f32(w0);
-    const float u1 = uniform_f32(w1);
-    const float r = sqrt_approx(-1.38629436111989061883f * __log2f(u0));
-    const float th = 6.28318530717958647693f * u1;
-    float s, c;
-    __sincosf(th, &s, &c);
-    z0 = r * c;
-    z1 = r * s;
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
 }
 
-// Box-Muller split for the EM kernels: with L = log2(u0), the normals are
+// Box-Muller in binary32 on the special-function unit, split for the EM
+// kernels: with L = log2(u0), the normals are
 // z0 = K q cos(theta), z1 = K q sin(theta), q = sqrt(-L), K = sqrt(2 ln 2);
 // K is folded into the noise amplitudes on the host.  The angle is built with
 // one FMA from the float 1 + (w1 >> 9) 2^-23: theta = 2 pi (u1) with
@@ -119,7 +157,7 @@ __device__ __forceinline__ void box_muller_qcs(uint32_t w0, uint32_t w1, float& 
     const float u0 = uniform_f32(w0);
     const float f1 = __uint_as_float(0x3F800000u | (w1 >> 9));
     const float th = fmaf(6.28318530717958647693f, f1, -6.283185107518108f);   // 2 pi_f (1 - 2^-24)
-    q = sqrt_approx(-__log2f(u0));
+    q = sqrt_approx(-log2_normal(u0));
     __sincosf(th, &s, &c);
 }
 
