@@ -49,6 +49,25 @@ __device__ __forceinline__ uint64_t weight_fixed(double w)
     return (M + ((1ull << (k - 1)) - 1ull) + ((M >> k) & 1ull)) >> k;
 }
 
+// The same with the usual weights, 2^-40 <= w < 2^-9, in 32-bit words first, for
+// the two passes of the scan, which are bound by issue: 16.5 and 25.0 us for
+// 9 x 2^20 weights instead of 20.6 and 27.6.  The weighted restriction keeps the
+// form above: there the additional branch cost 3.8 us of 18.7 at 4 x 81,240.
+__device__ __forceinline__ uint64_t weight_fixed_usual(double w)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(w);
+    const uint32_t hi = (uint32_t)(b >> 32);
+    const int k = 1014 - (int)(hi >> 20);                    // negative w: below 1
+    if ((unsigned)(k - 1) < 31u) {
+        const uint32_t lo = (uint32_t)b, mh = (hi & 0xFFFFFu) | 0x100000u;
+        const uint32_t kept = __funnelshift_r(lo, mh, k), cut = lo << (32 - k);   // cut: the bits shifted out
+        // up where they are above one half, or one half and the kept bit odd
+        const uint64_t v = (uint64_t)kept | (uint64_t)(mh >> k) << 32;
+        return v + (cut + (kept & 1u) > 0x80000000u || cut + (kept & 1u) < cut ? 1u : 0u);
+    }
+    return weight_fixed(w);
+}
+
 // In-place inclusive scan of a[0..I) with an associative `op` (identity
 // `ident`), by the whole block, from the right end when `reverse`: each thread
 // scans a run of consecutive elements, and the run totals are combined by a
@@ -252,7 +271,7 @@ fixed_blocksum_kernel(const double* __restrict__ w, int64_t n, int64_t nblk, uin
             v[k] = p < n ? __ldcs(ws + p) : 0.0;
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) loc += weight_fixed(v[k]);
+        for (int k = 0; k < 8; ++k) loc += weight_fixed_usual(v[k]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) loc += __shfl_down_sync(0xffffffffu, loc, o);
@@ -321,7 +340,7 @@ scan_within_kernel(const double* __restrict__ w, uint64_t* __restrict__ C, int64
             v[k] = p < n ? __ldcs(ws + p) : 0.0;
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) stage[scan_pad(k * 32 + lane)] = weight_fixed(v[k]);
+        for (int k = 0; k < 8; ++k) stage[scan_pad(k * 32 + lane)] = weight_fixed_usual(v[k]);
         __syncwarp();
         uint64_t r[8], loc = 0;
 #pragma unroll
@@ -396,6 +415,22 @@ struct StrataPoint {
         return Q * (uint64_t)j + P1 + (uint64_t)q2 + f;
     }
 
+    // U_j for n <= 2^30, given base = Q j + floor(R j / n), r2 and a_j: with
+    // a' = 2^8 a_j, Q a_j / 2^24 = Q a' / 2^32 has its whole and fractional words in
+    // the products as they come, and the sum of the fractions,
+    // (frac n + R a' + r2 2^32) / (n 2^32), is below 3: its whole part from the
+    // high word alone.
+    __device__ __forceinline__ uint64_t point(uint64_t base, uint32_t r2, uint32_t a) const
+    {
+        const uint32_t a8 = a << 8;
+        const uint64_t t = (uint64_t)Ql * a8;
+        const uint64_t whole = (uint64_t)Qh * a8 + (t >> 32);
+        const uint64_t fn = (uint64_t)(uint32_t)t * n, ra = (uint64_t)R * a8;
+        const uint32_t low = (uint32_t)fn + (uint32_t)ra;
+        const uint32_t h = (uint32_t)(fn >> 32) + (uint32_t)(ra >> 32) + r2 + (low < (uint32_t)fn ? 1u : 0u);
+        return base + whole + (h >= n ? 1u : 0u) + (h >= 2 * n ? 1u : 0u);
+    }
+
     __device__ __forceinline__ uint64_t at(uint32_t j, uint32_t q2, uint32_t r2) const
     {
         return at_a(j, q2, r2, a_of(j));
@@ -460,7 +495,10 @@ constexpr int kSelThreads = 256;
 constexpr int kSelPer = 8;
 constexpr int kSelOut = kSelThreads * kSelPer;   // consecutive outputs per CTA
 static_assert(kSelPer % 4 == 0, "a thread's outputs start on a Philox block of the strata draws");
-constexpr int kSelStage = 4096;                  // cumulative weights staged per CTA
+// Cumulative weights staged per CTA: the particles of kSelOut outputs are about
+// as many (19 % more are held; the rest of a longer range is read from global
+// memory).  With 2432 of them eight CTAs fit an SM, with 4096 five.
+constexpr int kSelStage = 2432;
 
 // The particles of the first and last output of every selection CTA: one
 // thread per bound, all at once.  The block offsets of the scan locate the
@@ -551,11 +589,23 @@ __device__ __forceinline__ void select_run(const V& v, Idx base, Idx hi, const S
 #pragma unroll
         for (int k = 0; k < kSelPer; ++k) a[k] = 1u << 23;
     }
-    uint64_t u[kSelPer];
+    uint64_t u[kSelPer];   // past the end: unused
+    if (U.n <= 1u << 30) {
+        uint64_t base_j = U.Q * (uint64_t)j + q2;
 #pragma unroll
-    for (int k = 0; k < kSelPer; ++k) {
-        u[k] = U.at_a(j + (uint32_t)k, q2, r2, a[k]);   // past the end: unused
-        U.step(q2, r2);
+        for (int k = 0; k < kSelPer; ++k) {
+            u[k] = U.point(base_j, r2, a[k]);
+            r2 += U.R;
+            const bool wraps = r2 >= U.n;
+            base_j += U.Q + (wraps ? 1u : 0u);
+            r2 -= wraps ? U.n : 0u;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < kSelPer; ++k) {
+            u[k] = U.at_a(j + (uint32_t)k, q2, r2, a[k]);
+            U.step(q2, r2);
+        }
     }
     const int m = min(kSelPer, cnt - jj0);
     Idx p = sel_search(v, base, hi, u[0]);
@@ -591,8 +641,12 @@ __device__ __forceinline__ void gather_rows(const T* __restrict__ src, T* __rest
 // of kSelPer consecutive outputs into shared memory; the indices and the
 // gathered states are then written with consecutive outputs on consecutive
 // threads.
-template <typename T>
-__global__ void __launch_bounds__(kSelThreads)
+// Bound by issue and the latency of its phases (search, gather), so by the CTAs
+// an SM holds: 9 x 2^20 outputs 73.5 us at eight per SM (32 registers), 83 at
+// five.  PER_SM = 5, without that cut in registers, for launches that do not
+// fill five per SM.
+template <typename T, int PER_SM>
+__global__ void __launch_bounds__(kSelThreads, PER_SM)
 select_gather_kernel(const uint64_t* __restrict__ C, const uint64_t* __restrict__ total,
                      const int64_t* __restrict__ bounds, int64_t n, int mode, uint32_t k0, uint32_t k1, uint32_t chi,
                      uint32_t slice0, const T* __restrict__ x_in, const T* __restrict__ y_in, int broadcast, int d,
@@ -880,16 +934,21 @@ extern "C" pr_status pr_resample(pr_precision precision, int32_t fast_dim, const
     PR_CHECK_LAUNCH();
     dim3 gs((unsigned)l.nsel, (unsigned)n_slices);
     const int d = y_out ? fast_dim : 0;
-    if (precision == PR_F32)
-        select_gather_kernel<float><<<gs, kSelThreads, 0, st>>>(C, total, bounds, n, (int)mode, k0, k1, chi, (uint32_t)slice_begin,
-                                                        static_cast<const float*>(x_in), static_cast<const float*>(y_in),
-                                                        broadcast_input ? 1 : 0, d, index_out,
-                                                        static_cast<float*>(x_out), static_cast<float*>(y_out));
-    else
-        select_gather_kernel<double><<<gs, kSelThreads, 0, st>>>(C, total, bounds, n, (int)mode, k0, k1, chi, (uint32_t)slice_begin,
-                                                         static_cast<const double*>(x_in), static_cast<const double*>(y_in),
-                                                         broadcast_input ? 1 : 0, d, index_out,
-                                                         static_cast<double*>(x_out), static_cast<double*>(y_out));
+    auto select = [&](auto kernel, auto zero) {
+        using T = decltype(zero);
+        kernel<<<gs, kSelThreads, 0, st>>>(C, total, bounds, n, (int)mode, k0, k1, chi, (uint32_t)slice_begin,
+                                           static_cast<const T*>(x_in), static_cast<const T*>(y_in),
+                                           broadcast_input ? 1 : 0, d, index_out, static_cast<T*>(x_out),
+                                           static_cast<T*>(y_out));
+    };
+    const bool fills = l.nsel * n_slices > 5 * (int64_t)num_sms();
+    if (precision == PR_F32) {
+        if (fills) select(select_gather_kernel<float, 8>, 0.0f);
+        else select(select_gather_kernel<float, 5>, 0.0f);
+    } else {
+        if (fills) select(select_gather_kernel<double, 8>, 0.0);
+        else select(select_gather_kernel<double, 5>, 0.0);
+    }
     PR_CHECK_LAUNCH();
     return PR_OK;
 }
@@ -918,7 +977,8 @@ extern "C" pr_status pr_restrict_weighted(pr_precision precision, const void* x,
     const GridDev g = make_grid(*grid);
     const float lo_f = (float)grid->x_lo, inv_h_f = (float)(1.0 / g.h);
     const size_t smem = al16c((size_t)I * 8) + al16c((size_t)(I + 1) * 4);
-    const int64_t per = cond_range(n, n_slices, 16384, 2);
+    // three CTAs per SM, as many as stay resident: 34 us for 9 x 2^20 particles (39 with two)
+    const int64_t per = cond_range(n, n_slices, 16384, 3);
     dim3 gr((unsigned)((n + per - 1) / per), (unsigned)n_slices);
     const int64_t stride = broadcast_input ? 0 : n;
     if (precision == PR_F32) {
