@@ -15,11 +15,12 @@
 // enter the binary64 sum once per 128 particles.
 //
 // Weighted sums and binary64 particles (moments_kernel): each order's term
-// enters its sum through one binary64 fused multiply-add (W v^(q-1) times v,
-// added with one rounding), and the running power takes one multiply: per
-// particle 2 max_order - 1 binary64 operations with weights, 2 max_order - 2
-// without (the first order adds v itself).  On GB300's narrow FP64 pipe that,
-// not HBM, bounds the pass.
+// enters its sum through one binary64 fused multiply-add.  Binary64 particles:
+// W v^(q-1) times v, the running power takes one multiply, 2 max_order - 1
+// binary64 operations per particle with weights, 2 max_order - 2 without (the
+// first order adds v itself).  Binary32 particles with weights: the exact v^2
+// comes from the integer units, 1, 2, 4, 5 operations for the orders up to 1..4.
+// On GB300's narrow FP64 pipe that, not HBM, bounds the pass.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -145,7 +146,7 @@ __device__ __forceinline__ bool run_exponent_ok(int e)
 
 // Bound by issue: 40 instructions per particle for the first two orders, 31 of
 // them binary32 additions and products.  49 x 2^20 particles, mean and second
-// moment: 67.6 us with the finishing kernel (211 us with binary64 terms), and
+// moment: 67.0 us with the finishing kernel (211 us with binary64 terms), and
 // closer to the exact sum (1.1e-16 instead of 3.6e-16).
 template <int Q>
 __global__ void __launch_bounds__(kMomThreads, Q <= 2 ? 6 : 4)
@@ -243,6 +244,29 @@ moments_f32_kernel(const float* __restrict__ v, int64_t stride, int64_t n, int64
     reduce_partials<Q>(acc, partial);
 }
 
+// The square of a binary32 number, exact in binary64, on the integer units: the
+// 48-bit product of the significands moved to the top of the fraction.
+// Subnormals, infinities and NaNs take the binary64 product.
+__device__ __forceinline__ double square_wide(float f)
+{
+    const uint32_t u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
+    if (e - 1u < 254u) {
+        const uint32_t m = (u & 0x7FFFFFu) | 0x800000u;
+        const uint64_t P = (uint64_t)m * m;              // f^2 = P 2^(2 (e - 150)), 2^46 <= P < 2^48
+        const uint32_t top = (uint32_t)(P >> 47);        // 1: from 2^47 on
+        return __longlong_as_double((long long)((P << (6 - top)) + ((uint64_t)(768 + 2 * e + top) << 52)));
+    }
+    if (u << 1 == 0u) return 0.0;
+    const double d = widen(f);
+    return d * d;
+}
+__device__ __forceinline__ double square_wide(double d) { return d * d; }
+
+// Bound by the binary64 pipe, 64 cycles per warp instruction.  Weighted binary32
+// values take Q of its instructions per particle for the first two orders (the
+// exact square comes from the integer units) and Q + 1 above, 2 Q - 1 with a
+// multiply per power, and round less often.  31 x 2,164,802 values, 3 orders: 476 us
+// instead of 603; 16 x 607,350, 4 orders: 100 us instead of 136.
 template <typename T, int Q, bool W>
 __global__ void __launch_bounds__(kMomThreads)
 moments_kernel(const T* __restrict__ v, int64_t stride, const double* __restrict__ w, int64_t n, int64_t per_block,
@@ -269,6 +293,17 @@ moments_kernel(const T* __restrict__ v, int64_t stride, const double* __restrict
         for (int k = 0; k < kMomUnroll; ++k) {
             if (p0 + (int64_t)k * kMomThreads >= e) break;
             const double x = widen(xv[k]);
+            if constexpr (W && Q >= 2 && sizeof(T) == 4) {
+                const double xx = square_wide(xv[k]);
+                acc[0] = fma(wv[k], x, acc[0]);
+                acc[1] = fma(wv[k], xx, acc[1]);
+                if constexpr (Q >= 3) {
+                    const double wxx = wv[k] * xx;
+                    acc[2] = fma(wxx, x, acc[2]);
+                    if constexpr (Q >= 4) acc[3] = fma(wxx, xx, acc[3]);
+                }
+                continue;
+            }
             double t;                     // W x^q before order q + 1
             int q0;
             if (W) {

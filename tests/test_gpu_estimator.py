@@ -5,6 +5,7 @@ sizes and several slices.  Every term is the same binary64 product on both
 sides; only the order of the additions differs, so the tolerance is a few
 units of rounding of the sum of absolute terms."""
 import math
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -208,3 +209,29 @@ def test_non_finite_values(L, bad, where):
         with np.errstate(invalid="ignore"):
             want = [np.sum(x.astype(np.float64) ** (q + 1)) for q in range(order)]
         np.testing.assert_array_equal(out.cpu().numpy()[0], want)
+
+
+@pytest.mark.parametrize("order", [2, 3, 4])
+def test_weighted_binary32_terms(L, order):
+    """One particle per slice: the first two orders' terms w v and w v^2 carry a
+    single rounding, the next two one more (3 units of 2^-53 allowed).  The
+    significands sit at the edges of the exact square (2^23, 2^24 - 1, either
+    side of sqrt 2), the exponents at both ends; subnormals and zeros."""
+    m = np.concatenate([[1 << 23, (1 << 24) - 1, (1 << 23) + 1, 11863283, 11863284],
+                        np.random.default_rng(3).integers(1 << 23, 1 << 24, 59)]).astype(np.float64)
+    v = np.concatenate([np.ldexp(m, e) for e in (-149, -148, -100, -30, -24, 0, 20, 104)]
+                       + [[0.0, -0.0, 2.0 ** -149, -(2.0 ** -127), 3.0 * 2.0 ** -149]])
+    v[1::3] *= -1.0
+    v = v.astype(np.float32)
+    rng = np.random.default_rng(4)
+    w = rng.random(v.size) * np.exp2(rng.integers(-40, 3, v.size))
+    w[5::17] *= -1.0
+    got = _gpu_moments(L, L.PR_F32, torch.from_numpy(v).to(DEV).reshape(-1, 1), 1,
+                       torch.from_numpy(w).to(DEV).reshape(-1, 1), 1, v.size, order)
+    for q in range(1, order + 1):
+        for i in range(v.size):
+            exact = Fraction(float(w[i])) * Fraction(float(v[i])) ** q
+            if q <= 2:
+                assert got[i, q - 1] == float(exact), (q, v[i], w[i])
+            else:
+                assert abs(Fraction(float(got[i, q - 1])) - exact) <= 3 * abs(exact) / 2 ** 53 + Fraction(1, 2 ** 1070)
