@@ -409,6 +409,17 @@ __device__ __forceinline__ void normals_f64(uint32_t w0, uint32_t w1, const Norm
 }
 
 // One step of a d = 1 family from its two normals.
+// sum / d, the same bits, from inv = 1 / d rounded: the quotient's residual from
+// one fused multiply-add corrects it to the rounded quotient (Markstein 1990).
+// Three binary64 instructions of 64 cycles instead of the division's nine.
+__device__ __forceinline__ double mean_f64(double sum, double d, double inv)
+{
+    const double q = sum * inv;
+    const uint32_t e = ((uint32_t)__double2hiint(q) >> 20) & 0x7FFu;
+    if (e - 123u < 1800u) return fma(fma(-q, d, sum), inv, q);   // 2^-900 <= |q| < 2^900
+    return sum / d;
+}
+
 template <int KIND>
 __device__ __forceinline__ void em_step_f64(const FineArgs& a, double& x, double& y, double z0, double z1)
 {
@@ -489,6 +500,7 @@ fine_f64_kernel(FineArgs a, FineSmemOffsets so, int flags)
             }
         } else {
             const int Q = 1 + D;
+            const double inv_D = 1.0 / (double)D;
             for (int m = 0; m < a.steps; ++m) {
                 double z[PR_MAX_FAST_DIM + 3];
                 // F full blocks per step, then the step's T = Q mod 4 normals from
@@ -509,7 +521,7 @@ fine_f64_kernel(FineArgs a, FineSmemOffsets so, int flags)
                 }
                 double ysum = 0.0;
                 for (int j = 0; j < D; ++j) ysum += y[j];
-                const double f = slow_force<1>(x, ysum / (double)D, a.lam);
+                const double f = slow_force<1>(x, mean_f64(ysum, (double)D, inv_D), a.lam);
                 const double xn = x - f * a.drift_dt + a.sx * z[0];
                 for (int j = 0; j < D; ++j) y[j] = y[j] - (y[j] - x) * a.relax + a.sy * z[1 + j];
                 x = xn;
