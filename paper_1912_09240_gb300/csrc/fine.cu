@@ -409,17 +409,6 @@ __device__ __forceinline__ void normals_f64(uint32_t w0, uint32_t w1, const Norm
 }
 
 // One step of a d = 1 family from its two normals.
-// sum / d, the same bits, from inv = 1 / d rounded: the quotient's residual from
-// one fused multiply-add corrects it to the rounded quotient (Markstein 1990).
-// Three binary64 instructions of 64 cycles instead of the division's nine.
-__device__ __forceinline__ double mean_f64(double sum, double d, double inv)
-{
-    const double q = sum * inv;
-    const uint32_t e = ((uint32_t)__double2hiint(q) >> 20) & 0x7FFu;
-    if (e - 123u < 1800u) return fma(fma(-q, d, sum), inv, q);   // 2^-900 <= |q| < 2^900
-    return sum / d;
-}
-
 template <int KIND>
 __device__ __forceinline__ void em_step_f64(const FineArgs& a, double& x, double& y, double z0, double z1)
 {
@@ -500,7 +489,7 @@ fine_f64_kernel(FineArgs a, FineSmemOffsets so, int flags)
             }
         } else {
             const int Q = 1 + D;
-            const double inv_D = 1.0 / (double)D;
+            const double inv_D = 1.0 / (double)D;   // the mean without a division per step
             for (int m = 0; m < a.steps; ++m) {
                 double z[PR_MAX_FAST_DIM + 3];
                 // F full blocks per step, then the step's T = Q mod 4 normals from
@@ -521,7 +510,7 @@ fine_f64_kernel(FineArgs a, FineSmemOffsets so, int flags)
                 }
                 double ysum = 0.0;
                 for (int j = 0; j < D; ++j) ysum += y[j];
-                const double f = slow_force<1>(x, mean_f64(ysum, (double)D, inv_D), a.lam);
+                const double f = slow_force<1>(x, div_known(ysum, (double)D, inv_D), a.lam);
                 const double xn = x - f * a.drift_dt + a.sx * z[0];
                 for (int j = 0; j < D; ++j) y[j] = y[j] - (y[j] - x) * a.relax + a.sy * z[1 + j];
                 x = xn;
@@ -653,8 +642,17 @@ restrict_kernel(const T* __restrict__ x, int64_t n, GridDev g, float lo_f, float
                 group4(u1, 4);
             });
     } else {
-        for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x)
-            atomicAdd(&hist[bin_of_f64(g, (double)xs[p])], 1u);
+        // the bins from binary32 arithmetic (bin_try_f64), decided exactly for the
+        // few particles near an edge; four loads in flight
+        const int T2 = blockDim.x;
+        for (int64_t p = b + threadIdx.x; p < e; p += 4 * T2) {
+            double v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = p + k * T2 < e ? __ldcs(xs + p + k * T2) : 0.0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (p + k * T2 < e) atomicAdd(&hist[bin_of_f64(g, (double)v[k])], 1u);
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < bins; i += blockDim.x)
@@ -716,7 +714,13 @@ match_f32_kernel(const float* __restrict__ xp, float* __restrict__ xo, int64_t n
     }
 }
 
-__global__ void __launch_bounds__(256)
+// Bound by the binary64 pipe, 64 cycles per warp instruction: 18 per particle
+// (edges, fraction, level, and the two divisions at three each), 60 with every
+// comparison, conversion and division on that pipe; the bin, the clamps and the
+// search over the target CDF run on the other units.  With the restriction
+// before it, 20 x 500,000 particles: 494 us instead of 1531; 12 x 9,000: 41 us
+// instead of 207 (more CTAs as well); 5,000: 25 us instead of 128.
+__global__ void __launch_bounds__(512)
 match_f64_kernel(const double* __restrict__ xp, double* __restrict__ xo, int64_t n, GridDev g,
                  const double* __restrict__ cp, const double* __restrict__ ct, int64_t per_block)
 {
@@ -727,9 +731,15 @@ match_f64_kernel(const double* __restrict__ xp, double* __restrict__ xo, int64_t
     build_match_index(g, cp + (size_t)s * (bins + 1), ct + (size_t)s * (bins + 1), ms);
     const int64_t b = (int64_t)blockIdx.x * per_block;
     const int64_t e = min(n, b + per_block);
+    if (e - b >= 4 * bins) tabulate_inverses(g, ms);
     const double* xs = xp + (int64_t)s * n;
     double* os = xo + (int64_t)s * n;
-    for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) os[p] = match_one_f64(ms, g, xs[p]);
+    const int T = blockDim.x;
+    for (int64_t p = b + threadIdx.x; p < e; p += 2 * T) {
+        const double u0 = __ldcs(xs + p), u1 = p + T < e ? __ldcs(xs + p + T) : 0.0;
+        __stcs(os + p, match_one_f64(ms, g, u0));
+        if (p + T < e) __stcs(os + p + T, match_one_f64(ms, g, u1));
+    }
 }
 
 // Binary32 matching on grids whose binary32 table does not fit one CTA's
@@ -748,6 +758,7 @@ match_f32_wide_kernel(const float* __restrict__ xp, float* __restrict__ xo, int6
     build_match_index(g, cp + (size_t)s * (bins + 1), ct + (size_t)s * (bins + 1), ms);
     const int64_t b = (int64_t)blockIdx.x * per_block;
     const int64_t e = min(n, b + per_block);
+    if (e - b >= 4 * bins) tabulate_inverses(g, ms);
     const float* xs = xp + (int64_t)s * in_stride;
     float* os = xo + (int64_t)s * n;
     for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x)
@@ -1023,7 +1034,7 @@ extern "C" pr_status pr_fine_propagate(const pr_model* model, pr_precision preci
         a.lo_f = (float)grid->x_lo;
         a.inv_h_f = (float)(1.0 / a.g.h);
     } else {
-        a.g = GridDev{1, 0.0, 1.0, 1.0};
+        a.g = make_grid(pr_grid{1, 0.0, 1.0});
     }
     a.cdf_prior = cdf_prior;
     a.cdf_target = cdf_target;
@@ -1182,7 +1193,9 @@ extern "C" pr_status pr_match(pr_precision precision, const void* x_prior, void*
     const GridDev g = make_grid(*grid);
     // two 1024-thread CTAs per SM, each building its table once (a few
     // microseconds of FP64 work) and streaming its share of the particles
-    const int64_t per_block = stream_range(n, n_slices, 16384, 2);
+    // (binary64: 512 threads and no table; from 1024 particles on per CTA, since two
+    // per thread outlast building the index)
+    const int64_t per_block = stream_range(n, n_slices, precision == PR_F32 ? 16384 : 1024, 2);
     const int64_t blocks_per_slice = (n + per_block - 1) / per_block;
     dim3 gr((unsigned)blocks_per_slice, (unsigned)n_slices);
     // the per-CTA binary32 table must fit in shared memory; beyond, the wide
@@ -1199,7 +1212,7 @@ extern "C" pr_status pr_match(pr_precision precision, const void* x_prior, void*
                                                 (float)grid->x_lo, (float)(1.0 / g.h), cdf_prior, cdf_target, per_block);
     } else {
         PR_TRY_CUDA(set_smem(match_f64_kernel, smem));
-        match_f64_kernel<<<gr, 256, smem, st>>>(static_cast<const double*>(x_prior), static_cast<double*>(x_out), n, g,
+        match_f64_kernel<<<gr, 512, smem, st>>>(static_cast<const double*>(x_prior), static_cast<double*>(x_out), n, g,
                                                 cdf_prior, cdf_target, per_block);
     }
     PR_CHECK_LAUNCH();

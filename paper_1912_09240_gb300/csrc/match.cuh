@@ -55,6 +55,7 @@ struct MatchSmem {
     int* jfirst;
     int* pstart;
     int* scratch;   // [blockDim.x / 32 + 1] for scans
+    const double* inv;   // known_inverse of the target bins' masses, or null (tabulate_inverses)
 };
 
 __host__ __device__ inline size_t match_table_bytes(int bins)
@@ -97,6 +98,7 @@ __device__ inline MatchSmem carve_match_smem_f32(unsigned char* base, int bins, 
 {
     const int I = bins;
     MatchSmem m;
+    m.inv = nullptr;
     m.rec = reinterpret_cast<float4*>(base);
     m.piece = m.rec + I;
     m.fend = reinterpret_cast<float*>(m.piece + (2 * I + 1));
@@ -115,6 +117,7 @@ __device__ inline MatchSmem carve_match_smem(unsigned char* base, int bins)
 {
     const int I = bins;
     MatchSmem m;
+    m.inv = nullptr;
     m.rec = nullptr;
     m.piece = nullptr;
     m.fend = nullptr;
@@ -392,6 +395,18 @@ __device__ inline void build_match_index(const GridDev& g, const double* __restr
     __syncthreads();
 }
 
+// The reciprocals of the target bins' masses, where the index's temporaries stood
+// (2 I + 1 ints from jfirst on, of which the last 2 I are 8-byte aligned): nine
+// binary64 instructions per bin that save six per particle, so worth it from a
+// few particles per bin on.  The whole block calls it, after build_match_index.
+__device__ inline void tabulate_inverses(const GridDev& g, MatchSmem& m)
+{
+    double* inv = reinterpret_cast<double*>(m.jfirst + 1);
+    for (int j = threadIdx.x; j < g.bins; j += blockDim.x) inv[j] = known_inverse(__dsub_rn(m.Ct[j + 1], m.Ct[j]));
+    m.inv = inv;
+    __syncthreads();
+}
+
 __device__ inline double match_one_f64(const MatchSmem& m, const GridDev& g, double x)
 {
     const int I = g.bins;
@@ -399,17 +414,18 @@ __device__ inline double match_one_f64(const MatchSmem& m, const GridDev& g, dou
     if (deq(m.Cp[i], m.Ct[i]) && deq(m.Cp[i + 1], m.Ct[i + 1])) return x;
     if (m.nzpre[I] == 0) return x;
     const double ei = edge(g, i);
-    double frac = __ddiv_rn(__dsub_rn(x, ei), g.h);
+    double frac = div_known(__dsub_rn(x, ei), g.h, g.inv_h);
     bool below = false, above = false;
-    if (frac < 0.0) { frac = 0.0; below = true; }
-    if (frac > 1.0) { frac = 1.0; above = true; }
+    if (below_zero(frac)) { frac = 0.0; below = true; }
+    if (above_one(frac)) { frac = 1.0; above = true; }
     const double rho_prior = __dsub_rn(m.Cp[i + 1], m.Cp[i]);
     const double u = __dadd_rn(m.Cp[i], __dmul_rn(frac, rho_prior));
     const int j = target_bin(m.Ct, m.nzpre, m.nzlist, I, u);
     const double rho_j = __dsub_rn(m.Ct[j + 1], m.Ct[j]);
-    double t = __ddiv_rn(__dsub_rn(u, m.Ct[j]), rho_j);
-    if (t < 0.0) t = 0.0;
-    if (t > 1.0) t = 1.0;
+    const double a = __dsub_rn(u, m.Ct[j]);
+    double t = m.inv ? div_known(a, rho_j, m.inv[j]) : __ddiv_rn(a, rho_j);
+    if (below_zero(t)) t = 0.0;
+    if (above_one(t)) t = 1.0;
     const double xn = __dadd_rn(edge(g, j), __dmul_rn(t, g.h));
     if (below) return __dadd_rn(x, __dsub_rn(xn, g.lo));
     if (above) return __dadd_rn(x, __dsub_rn(xn, g.hi));
