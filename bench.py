@@ -44,15 +44,15 @@ UNIT = "particle-steps/s"
 WORKLOAD = workloads.DOUBLE_WELL
 # Thread-instructions per particle-step of the binary32 fine kernel (d = 1,
 # 4 particles per thread): ncu smsp__inst_executed.sum x 32 over the
-# particle-steps of the launch, double-well workload at 2^16 and at 2^20
-# particles x 9 slices x 1000 steps (the same count at both sizes).
-INST_PER_PARTICLE_STEP = 41.58
+# particle-steps of the launch, double-well workload at 2^20 particles x 9
+# slices x 1000 steps.
+INST_PER_PARTICLE_STEP = 37.65
 # DRAM bytes per particle per slice of that kernel, read + write (ncu
 # dram__bytes_read.sum + dram__bytes_write.sum of the 9-slice launch at 2^21
 # particles, inputs larger than L2, scaled by particle-slices to the full
 # launch); the algorithmic figure is
 # 16 B (x and y read once and written once, binary32).
-TRAFFIC_BYTES_PER_PARTICLE_SLICE = 13.75
+TRAFFIC_BYTES_PER_PARTICLE_SLICE = 13.87
 SMS = 152
 ISSUE_LANES_PER_SM_CLK = 4 * 32       # 4 sub-partitions x one 32-wide warp instruction per clock
 
@@ -265,8 +265,8 @@ def _unfused_leg(L, solver, w, stream, hbm_peak):
     out = {"restrict": {"ms": t_r, "algorithmic_bytes": rb, "gbs": rb / t_r / 1e6},
            "match": {"ms": t_m, "algorithmic_bytes": mb, "gbs": mb / t_m / 1e6},
            "moments_q2": {"ms": t_e, "algorithmic_bytes": rb, "gbs": rb / t_e / 1e6,
-                          "fp64_ops_per_particle": 2,
-                          "fp64_ops_per_s": 2.0 * n * S / t_e / 1e-3},
+                          "fp32_ops_per_particle": 29,
+                          "fp32_ops_per_s": 29.0 * n * S / t_e / 1e-3},
            "coarse_fp_us": 1e3 * t_c, "serial_sweep_us": 1e3 * t_u,
            "note": f"{S} slices x {n} binary32 particles; coarse step on {K} states of {w.bins} bins; "
                    f"sweep over {K} slices"}

@@ -308,9 +308,11 @@ pr_status pr_restrict_weighted(pr_precision precision, const void* x, int32_t br
  * of each slice's ensemble (the slow variable, or one fast component):
  *   out[s][q-1] = sum_p W^p (v^p)^q,
  * W^p = w[s][p] when w is given, else 1/n (taken as the sum divided by n).
- * Binary64 accumulation (each term added by one fused multiply-add) in a
- * fixed order that depends only on n and n_slices, so repeated calls return
- * the same bits.
+ * Accumulated with at least binary64's precision (binary32 values without
+ * weights: error-free binary32 words, entered into binary64 sums every 128
+ * values; otherwise each term by one binary64 fused multiply-add) in a fixed
+ * order that depends only on n and n_slices, so repeated calls return the same
+ * bits.
  *   v (device) precision as given; slice s starts slice_stride elements after
  *     slice s-1 (n for x[n_slices][n]; fast_dim * n for component c of
  *     y[n_slices][fast_dim][n], passing y + c * n); slice_stride >= n when

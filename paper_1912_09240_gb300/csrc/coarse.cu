@@ -3,8 +3,9 @@
 // mm_sequential) with the iterators of Section 4, and the W1 distance.
 //
 // Everything here is FP64.  The macroscopic states are short (I <= 4096 bins,
-// the serial update I <= 1024), so the work is latency-bound: one CTA per
-// state vector, and one CTA for the serial sweep over the slices.  Operations
+// the serial update I <= 1024), so the work is latency-bound: a CTA or a
+// cluster per state vector, and one cluster for the serial sweep over the
+// slices.  Operations
 // that decide exactness (edges, quantile interpolation, the monotone repair,
 // reading the CDF back at the edges) are written with explicitly rounded
 // intrinsics so that no multiply-add is fused.
