@@ -231,6 +231,11 @@ __device__ __forceinline__ void coarse_rows(const double* __restrict__ P, int I,
 // All in shared memory; every thread of a kCoarseThreads block calls it.
 // ---------------------------------------------------------------------------
 
+constexpr int kShareBins = 256;   // beyond, the division of the CDF is split over the cluster
+
+// The cluster's CTAs meet once in it, or twice above kShareBins: a caller that
+// comes back lets them meet again in between (the next call writes into `mp` of
+// CTAs that may still read it).
 template <int CL = 1>
 __device__ inline void coarse_apply_block(const double* __restrict__ P, int I, const double* cdf_in,
                                           double* out, double* mass, double* mp, double* wsum,
@@ -264,7 +269,7 @@ __device__ inline void coarse_apply_block(const double* __restrict__ P, int I, c
     // every CTA divides all of them where that takes less than the exchange
     // (I / 32 divisions of 9 binary64 instructions on four sub-partitions, about
     // 1000 cycles for the exchange)
-    const bool split = CL > 1 && I > 256;
+    const bool split = CL > 1 && I > kShareBins;
     const int q0 = split ? d.lo(I - 1) : 0, q1 = split ? d.hi(I - 1) : I - 1;
     for (int r = q0 + threadIdx.x; r < q1; r += blockDim.x) {
         const double v = total > 0.0 ? __ddiv_rn(mp[r], total) : 0.0;
@@ -833,7 +838,10 @@ __device__ inline void serial_sweep(unsigned char* usm, const double* __restrict
             cur[i] = v;
             if (writer) next[(size_t)(n + 1) * (I + 1) + i] = v;
         }
-        __syncthreads();
+        // an exchange has followed the coarse step's first one, unless the grid is
+        // small and the iterator has none
+        if (iterator != PR_ITER_QUANTILE && I <= kShareBins) d.sync();
+        else __syncthreads();
     }
     if (threadIdx.x == 0 && status && writer) *status = js.flag[1] ? PR_ERR_NUMERIC : PR_OK;
     d.sync();   // no CTA leaves while another may still write into its shared memory
