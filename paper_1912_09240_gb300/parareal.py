@@ -390,8 +390,10 @@ class PararealSolver:
         first use (capture enqueues nothing; the replay does the work)."""
         p = self._swaps % 2
         s = self._s()
+        # behind an eager iteration's work on the side streams (iteration 0 of a
+        # solver whose graphs exist already from an earlier run)
+        self.join()
         if self._graphs[p] is None:
-            self.join()
             cs = torch.cuda.Stream(self.device)
             cs.wait_stream(s)
             g = torch.cuda.CUDAGraph()
