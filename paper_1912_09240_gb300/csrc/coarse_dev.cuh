@@ -233,9 +233,10 @@ __device__ __forceinline__ void coarse_rows(const double* __restrict__ P, int I,
 
 constexpr int kShareBins = 256;   // beyond, the division of the CDF is split over the cluster
 
-// The cluster's CTAs meet once in it, or twice above kShareBins: a caller that
-// comes back lets them meet again in between (the next call writes into `mp` of
-// CTAs that may still read it).
+// The cluster's CTAs meet once in it, or twice above kShareBins.  After one
+// meeting a CTA may return while others still scan and divide their `mp`: until
+// they have met again it stores nothing into `mp` of theirs, nor into memory
+// that overlaps it.
 template <int CL = 1>
 __device__ inline void coarse_apply_block(const double* __restrict__ P, int I, const double* cdf_in,
                                           double* out, double* mass, double* mp, double* wsum,
@@ -339,11 +340,19 @@ __device__ __forceinline__ void quantiles(const GridDev& g, const double* edges,
     qm = qp = q;
 }
 
+// Remote stores (Dist::share) go into mp, counted, kq and the CDFs `out` only.
+// Between an exchange's barrier and the next exchange the CTAs of a cluster run
+// apart, so the target of the next one must overlap nothing that a CTA still
+// uses in between (its own part of the target apart):
+//   mp       behind the barrier that ends the slice before (see serial_sweep)
+//   counted  behind share(mp); in between mass, mp, wsum and the CDFs
 struct JqSmem {
-    double* levels;   // [3(I+1)]
+    double* levels;   // [3(I+1)]; before the iterator the coarse step's mass | mp [I] each
+    double *mass, *mp;
+    unsigned long long* counted;   // [3(I+1)]  counts per value, in ibuf (the repair comes later)
     double* kq;       // [6(I+1)]  counts of the merged levels, then knots
     double* bsum;     // [6(I+1)]  merged levels | counts of the distinct ones, then scratch of the repair
-    int* ibuf;        // [6(I+1)]  segment starts, then sizes of pooled blocks
+    int* ibuf;        // [6(I+1)]  counts per value, then segment starts, then sizes of pooled blocks
     int* bpos;        // [6(I+1)]  segments to pool | pooled blocks
     int* flag;        // [0]: level count, [1]: input not a CDF, [2]: segments to pool, [3]: pooled blocks
     double* wsum;     // [kWsum]
@@ -356,16 +365,19 @@ __host__ __device__ inline size_t jq_smem_bytes(int bins)
     return (M + 2 * M + 2 * M + kWsum + (size_t)(bins + 1)) * sizeof(double) + (4 * M + 4) * sizeof(int);
 }
 
-__device__ inline JqSmem carve_jq(unsigned char* base, int bins)
+__host__ __device__ inline JqSmem carve_jq(unsigned char* base, int bins)
 {
     const int M = 3 * (bins + 1);
     JqSmem j;
     j.levels = reinterpret_cast<double*>(base);
+    j.mass = j.levels;
+    j.mp = j.levels + bins;
     j.kq = j.levels + M;
     j.bsum = j.kq + 2 * M;
     j.wsum = j.bsum + 2 * M;
     j.edges = j.wsum + kWsum;
     j.ibuf = reinterpret_cast<int*>(j.edges + bins + 1);
+    j.counted = reinterpret_cast<unsigned long long*>(j.ibuf);
     j.bpos = j.ibuf + 2 * M;
     j.flag = j.bpos + 2 * M;
     return j;
@@ -490,7 +502,7 @@ __device__ inline void quantile_iterate_block(const GridDev& g, int qmode, const
     //    with each element how many values of A, B and C lie below it (exact
     //    for the first of equal elements) into kq
     unsigned long long* below = reinterpret_cast<unsigned long long*>(s.kq);
-    unsigned long long* counted = reinterpret_cast<unsigned long long*>(s.levels);   // (the levels come later)
+    unsigned long long* counted = s.counted;
     {
         const int m0 = d.lo(M), m1 = d.hi(M);   // this CTA's share
         for (int k = m0 + threadIdx.x; k < m1; k += 2 * T) {
@@ -810,8 +822,6 @@ __device__ inline void serial_sweep(unsigned char* usm, const double* __restrict
     double* Cb = Bb + (I + 1);
     double* Ob = Cb + (I + 1);
     JqSmem js = carve_jq(reinterpret_cast<unsigned char*>(Ob + (I + 1)), I);
-    double* mass = js.levels;       // coarse scratch aliases the level list
-    double* mp = js.levels + I;
     if (threadIdx.x == 0) js.flag[1] = 0;
     fill_edges(g, js);
     for (int i = threadIdx.x; i <= I; i += blockDim.x) {
@@ -820,7 +830,7 @@ __device__ inline void serial_sweep(unsigned char* usm, const double* __restrict
     }
     d.sync();   // every CTA of the cluster runs before any writes into its shared memory
     for (int n = 0; n < K; ++n) {
-        coarse_apply_block<CL>(P, I, cur, Ab, mass, mp, js.wsum, d);
+        coarse_apply_block<CL>(P, I, cur, Ab, js.mass, js.mp, js.wsum, d);
         double* res = Ab;
         if (iterator != PR_ITER_NONE) {
             for (int i = threadIdx.x; i <= I; i += blockDim.x) {
@@ -838,8 +848,9 @@ __device__ inline void serial_sweep(unsigned char* usm, const double* __restrict
             cur[i] = v;
             if (writer) next[(size_t)(n + 1) * (I + 1) + i] = v;
         }
-        // an exchange has followed the coarse step's first one, unless the grid is
-        // small and the iterator has none
+        // the next slice stores into mp of CTAs that may still divide it, unless an
+        // exchange has followed the coarse step's first one (the quantile
+        // iterator's, or that of `out` on larger grids)
         if (iterator != PR_ITER_QUANTILE && I <= kShareBins) d.sync();
         else __syncthreads();
     }
