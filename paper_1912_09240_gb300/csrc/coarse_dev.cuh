@@ -346,14 +346,20 @@ __device__ __forceinline__ void quantiles(const GridDev& g, const double* edges,
 // uses in between (its own part of the target apart):
 //   mp       behind the barrier that ends the slice before (see serial_sweep)
 //   counted  behind share(mp); in between mass, mp, wsum and the CDFs
+//   kq       behind share(counted); in between counted, below, per, levels, bsum
+//            and the CDFs
+//   out      behind share(kq) (the coarse step's: share(mp)); in between none of
+//            its own kind
 struct JqSmem {
     double* levels;   // [3(I+1)]; before the iterator the coarse step's mass | mp [I] each
     double *mass, *mp;
     unsigned long long* counted;   // [3(I+1)]  counts per value, in ibuf (the repair comes later)
-    double* kq;       // [6(I+1)]  counts of the merged levels, then knots
+    unsigned long long* below;     // [3(I+1)]  counts of the merged levels, in bpos (likewise)
+    int* per;                      // [3(I+1) / 32 rounded up]  distinct levels per group of 32, in wsum
+    double* kq;       // [6(I+1)]  knots
     double* bsum;     // [6(I+1)]  merged levels | counts of the distinct ones, then scratch of the repair
     int* ibuf;        // [6(I+1)]  counts per value, then segment starts, then sizes of pooled blocks
-    int* bpos;        // [6(I+1)]  segments to pool | pooled blocks
+    int* bpos;        // [6(I+1)]  counts of the merged levels, then segments to pool | pooled blocks
     int* flag;        // [0]: level count, [1]: input not a CDF, [2]: segments to pool, [3]: pooled blocks
     double* wsum;     // [kWsum]
     double* edges;    // [I+1]  edge(g, i) (fill_edges)
@@ -379,6 +385,8 @@ __host__ __device__ inline JqSmem carve_jq(unsigned char* base, int bins)
     j.ibuf = reinterpret_cast<int*>(j.edges + bins + 1);
     j.counted = reinterpret_cast<unsigned long long*>(j.ibuf);
     j.bpos = j.ibuf + 2 * M;
+    j.below = reinterpret_cast<unsigned long long*>(j.bpos);
+    j.per = reinterpret_cast<int*>(j.wsum);
     j.flag = j.bpos + 2 * M;
     return j;
 }
@@ -485,7 +493,7 @@ __device__ inline void quantile_iterate_block(const GridDev& g, int qmode, const
     const int n1 = I + 1;
     const int M = 3 * n1;
     const int T = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = T >> 5;
-    int* per = s.bpos;   // counts per group of 32 (compactions)
+    int* per = s.per;
     if (threadIdx.x == 0) s.flag[2] = s.flag[3] = 0;
     // validity: in [0, 1] (NaN fails) and non-decreasing, by ordered keys
     const long long k0 = okey(0.0), k1 = okey(1.0);
@@ -500,8 +508,8 @@ __device__ inline void quantile_iterate_block(const GridDev& g, int qmode, const
     }
     // 1. sorted union of the 3(I+1) levels (stable merge by rank) into bsum, and
     //    with each element how many values of A, B and C lie below it (exact
-    //    for the first of equal elements) into kq
-    unsigned long long* below = reinterpret_cast<unsigned long long*>(s.kq);
+    //    for the first of equal elements) into below
+    unsigned long long* below = s.below;
     unsigned long long* counted = s.counted;
     {
         const int m0 = d.lo(M), m1 = d.hi(M);   // this CTA's share

@@ -29,6 +29,8 @@ int main(int argc, char** argv)
         show("mp", j.mp, 8 * (size_t)I);
         show("counted", j.counted, 8 * (size_t)M);
         show("kq", j.kq, 16 * (size_t)M);
+        show("below", j.below, 8 * (size_t)M);
+        show("per", j.per, 4 * (size_t)((M + 31) / 32));
         show("bsum", j.bsum, 16 * (size_t)M);
         show("wsum", j.wsum, 8 * (size_t)pr::kWsum);
         show("edges", j.edges, 8 * (size_t)(I + 1));
@@ -62,3 +64,13 @@ def _apart(places, target, others):
 def test_counts_exchanged_beside_the_coarse_step(layout, bins):
     """share(mp) .. share(counted): the coarse step's scan and division, the edges and the status flag."""
     _apart(layout[bins], "counted", ["mass", "mp", "wsum", "edges", "flag"])
+
+
+@pytest.mark.parametrize("bins", BINS)
+def test_knots_exchanged_beside_the_levels(layout, bins):
+    """share(counted) .. share(kq): merge, compaction and quantiles (which read `below`, not their own knots)."""
+    _apart(layout[bins], "kq", ["counted", "below", "per", "levels", "bsum", "wsum", "edges", "flag"])
+    _apart(layout[bins], "below", ["counted", "per", "levels", "bsum", "wsum", "edges", "flag"])
+    # the group counts fit the scratch that they stand in
+    p = layout[bins]
+    assert p["wsum"][0] <= p["per"][0] and p["per"][1] <= p["wsum"][1]
