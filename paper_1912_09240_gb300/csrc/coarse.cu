@@ -289,7 +289,7 @@ coarse_fp_kernel(const double* __restrict__ P, int I, const double* __restrict__
     const size_t v = blockIdx.x / CL;
     const double* src = cin + v * (I + 1);
     for (int i = threadIdx.x; i <= I; i += blockDim.x) in[i] = src[i];
-    __syncthreads();
+    d.sync();   // every CTA of the cluster runs before any writes into its shared memory
     coarse_apply_block<CL>(P, I, in, out, mass, mp, wsum, d);
     double* dst = cout + v * (I + 1);
     const int q0 = d.lo(I - 1), q1 = d.hi(I - 1);
