@@ -66,8 +66,9 @@ constexpr double kTailMass = 1e-10;
 // Block-level FP64 helpers (deterministic order for a fixed blockDim)
 // ---------------------------------------------------------------------------
 
-// Ordered 64-bit key of a non-NaN double: signed comparison of keys is
-// numeric comparison, and -0 and +0 both map to 0.
+// Ordered 64-bit key of a double: signed comparison of keys is numeric
+// comparison, and -0 and +0 both map to 0.  The keys of NaNs lie beyond those
+// of the infinities, on the side of their sign bit.
 __device__ __forceinline__ long long okey(double v)
 {
     const long long b = __double_as_longlong(v);
@@ -85,9 +86,22 @@ __device__ __forceinline__ float narrow(double v)
     return (float)v;
 }
 
-// The larger of two non-NaN doubles, on the integer units (a binary64
+// a > b and a <= b on the integer units, false where either is a NaN (a binary64
 // comparison takes the FP64 pipe, 64 cycles of a sub-partition).
-__device__ __forceinline__ double max_f64(double a, double b) { return okey(a) >= okey(b) ? a : b; }
+constexpr long long kKeyInf = 0x7FF0000000000000ll;
+__device__ __forceinline__ bool greater_f64(double a, double b)
+{
+    const long long x = okey(a), y = okey(b);
+    return x > y && x <= kKeyInf && y >= -kKeyInf;
+}
+__device__ __forceinline__ bool at_most_f64(double a, double b)
+{
+    const long long x = okey(a), y = okey(b);
+    return x <= y && x >= -kKeyInf && y <= kKeyInf;
+}
+
+// The larger of a (not a NaN) and b; a NaN in b is passed over.
+__device__ __forceinline__ double max_f64(double a, double b) { return greater_f64(b, a) ? b : a; }
 
 constexpr int kWsum = 56;   // doubles of the scratch `wsum` of the block-level helpers
 
@@ -221,7 +235,7 @@ __device__ __forceinline__ void coarse_rows(const double* __restrict__ P, int I,
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
         const int h = (b4 ? 1 : 0) + (b3 ? 2 : 0);   // the row of this lane's sum
-        if ((lane & 7) == 0 && h < R && r + h < r1) mp[r + h] = okey(v) > okey(kTailMass) ? v : 0.0;
+        if ((lane & 7) == 0 && h < R && r + h < r1) mp[r + h] = greater_f64(v, kTailMass) ? v : 0.0;
     }
 }
 
@@ -274,7 +288,7 @@ __device__ inline void coarse_apply_block(const double* __restrict__ P, int I, c
     const int q0 = split ? d.lo(I - 1) : 0, q1 = split ? d.hi(I - 1) : I - 1;
     for (int r = q0 + threadIdx.x; r < q1; r += blockDim.x) {
         const double v = total > 0.0 ? __ddiv_rn(mp[r], total) : 0.0;
-        out[r + 1] = dkey(v) < dkey(1.0) ? v : 1.0;
+        out[r + 1] = greater_f64(1.0, v) ? v : 1.0;
     }
     if (threadIdx.x == 0) {
         out[0] = 0.0;
@@ -335,8 +349,8 @@ __device__ __forceinline__ void quantiles(const GridDev& g, const double* edges,
     const double t = __ddiv_rn(__dsub_rn(p, F[lt - 1]), __dsub_rn(F[lt], F[lt - 1]));
     const double e0 = edges[lt - 1], e1 = edges[lt];
     double q = __dadd_rn(e0, __dmul_rn(t, g.h));
-    if (okey(q) <= okey(e0)) q = nextafter(e0, e1);
-    if (okey(q) >= okey(e1)) q = nextafter(e1, e0);
+    if (at_most_f64(q, e0)) q = nextafter(e0, e1);
+    if (at_most_f64(e1, q)) q = nextafter(e1, e0);
     qm = qp = q;
 }
 
@@ -432,7 +446,7 @@ static __device__ __noinline__ void pool_segment(double* kq, double* bsum, int* 
     auto above = [](double l, float lf, float l_n, double r, float rf, float r_n) {
         const float x = lf * r_n, y = rf * l_n, diff = x - y;
         if (fabsf(diff) > 0x1p-19f * fmaxf(fabsf(x), fabsf(y))) return diff > 0.0f;
-        return okey(__dmul_rn(l, (double)r_n)) > okey(__dmul_rn(r, (double)l_n));
+        return greater_f64(__dmul_rn(l, (double)r_n), __dmul_rn(r, (double)l_n));
     };
     do {
         const float qf = narrow(q);
@@ -735,8 +749,8 @@ __device__ inline void quantile_iterate_block(const GridDev& g, int qmode, const
                 v = __dadd_rn(pj, __dmul_rn(t, __dsub_rn(pn, pj)));
             }
         }
-        if (okey(v) < k0) v = 0.0;
-        if (okey(v) > k1 && !isnan(v)) v = 1.0;
+        if (greater_f64(0.0, v)) v = 0.0;   // (a NaN stays: the caller reports it)
+        if (greater_f64(v, 1.0)) v = 1.0;
         out[i] = v;
     }
     if (threadIdx.x == 0) {
