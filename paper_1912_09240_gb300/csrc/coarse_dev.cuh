@@ -431,9 +431,11 @@ __device__ __forceinline__ int warp_prefix_int(const int* per, int g)
 //
 // A serial chain, so what counts is its length: binary64 instructions take 64
 // cycles each, so the comparisons are first made in binary32, which decides
-// them exactly wherever the products differ by more than their rounding, and
-// one addition per merge is left.  (Not inlined: the sweep around it leaves it
-// no registers.)
+// them exactly wherever the products differ by more than their rounding (sums
+// cut to 2^-23, 2^-24 per product: far below the 2^-19 asked for, as long as
+// the larger product is 2^-100 at least, where what binary32 loses of smaller
+// numbers, up to 2^-149 per knot, does not matter either), and one addition per
+// merge is left.  (Not inlined: the sweep around it leaves it no registers.)
 static __device__ __noinline__ void pool_segment(double* kq, double* bsum, int* ibuf, int* n_blocks, int* blocks, int a,
                                           int nk)
 {
@@ -445,7 +447,8 @@ static __device__ __noinline__ void pool_segment(double* kq, double* bsum, int* 
     // mean(left) > mean(right)
     auto above = [](double l, float lf, float l_n, double r, float rf, float r_n) {
         const float x = lf * r_n, y = rf * l_n, diff = x - y;
-        if (fabsf(diff) > 0x1p-19f * fmaxf(fabsf(x), fabsf(y))) return diff > 0.0f;
+        const float top = fmaxf(fabsf(x), fabsf(y));
+        if (top >= 0x1p-100f && fabsf(diff) > 0x1p-19f * top) return diff > 0.0f;
         return greater_f64(__dmul_rn(l, (double)r_n), __dmul_rn(r, (double)l_n));
     };
     do {

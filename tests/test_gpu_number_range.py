@@ -1,6 +1,8 @@
-"""Infinities and NaNs in the coarse step and the iterators, whose comparisons
-run on the integer units: they decide as the floating comparisons do, whatever
-the sign bit of a NaN, so that a NaN reaches the caller's status."""
+"""The ends of the number range in the coarse step and the iterators.  Their
+comparisons run on the integer units and in binary32: with infinities and NaNs
+they decide as the floating comparisons do, whatever the sign bit of a NaN, so
+that a NaN reaches the caller's status, and on grids whose knots are below
+binary32's range as the binary64 products do."""
 import math
 
 import numpy as np
@@ -82,3 +84,17 @@ def test_coarse_step_of_what_is_no_cdf(L, bins, last):
         want[1 + np.argmax(full):] = 1.0
     want[-1] = 1.0
     np.testing.assert_array_equal(got, want)
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-36, 1e-40, 1e-42, 1e-44, 1e-46, 1e-60, 1e-300])
+@pytest.mark.parametrize("qmode", [0, 1])
+@pytest.mark.parametrize("bins", [64, 300, 700])
+def test_pooled_knots_below_the_range_of_binary32(L, scale, qmode, bins):
+    """Bit for bit the oracle's pooling, as on grids of ordinary size."""
+    lo, hi = -3.0 * scale, 3.0 * scale
+    for rows in ((_gauss(bins, 0.9, 0.5), _gauss(bins, -0.2, 0.4), _gauss(bins, 0.1, 0.9)),
+                 (_gauss(bins, 0.0, 0.2), _gauss(bins, 0.1, 0.9), _gauss(bins, 0.0, 1.2))):
+        got, st = _iterate(L, L.Grid(bins, lo, hi), qmode, rows)
+        assert st == 0
+        want = oracle.iterate(oracle.Grid(bins, lo, hi), *rows, oracle.ITER_QUANTILE, qmode)
+        np.testing.assert_array_equal(got, want)
