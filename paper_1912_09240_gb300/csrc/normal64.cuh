@@ -6,14 +6,18 @@
 // Euler-Maruyama step.  Here the pair is computed on the integer units in
 // 64-bit fixed point and only then turned into binary64, so that the pipe is
 // left to the step itself:
-//   radius  r(u0) = sqrt(-2 ln u0), 2^-60 units: a polynomial of degree 7 per
-//           segment (46 binades of u0 and 1 - u0 x 32), Horner with a 31-bit
-//           argument;
-//   angle   2 pi u1 = quarter turns + node + b: cos and sin of the 1024 nodes
-//           of a quarter turn in 2^-63 units, of b < 2^-9 from its series, and
-//           the addition formulas.
-// The normals are within 2^-57 of the exact ones (2^-58.5 rms), below the
-// rounding of a binary64 number of their size except where |z| < 2^-4.
+//   radius  r(u0) = sqrt(-2 ln u0): a polynomial of degree 7 per segment (46
+//           binades of u0 and 1 - u0 x 32), Horner with a 31-bit argument, in
+//           units of 2^-(60 + shift) that leave r 61 bits at least in every
+//           binade;
+//   angle   2 pi u1 reflected into an eighth of a turn = node + b: cos and sin of
+//           the 1024 nodes, of b < 2^-10.3 from its series, and the addition
+//           formulas.  The sine is a sum of positive terms there, kept in 96 bits
+//           and normalised to 63, so that it keeps its bits where it is small.
+// So the normals have the same relative error at every size, before the one
+// rounding to binary64 2^-59.3 rms and 2^-54.6 at most (at the first nodes, whose
+// sines are rounded to 2^-65), after it 2^-54.2 rms; a pair in absolute fixed
+// point lost its bits where it is small (2^-47.5 rms, 2^-41 below 2^-12).
 // Tables and constants: normal_tables.py (the header it writes is included by
 // the translation unit that holds the tables).
 #pragma once
@@ -24,10 +28,12 @@
 #define PR_CLZ(v) __clz((int)(v))
 #define PR_UMULHI(a, b) __umulhi((a), (b))
 #define PR_SMULHI(a, b) __mulhi((a), (b))
+#define PR_FUNNEL_L(lo, hi, n) __funnelshift_l((lo), (hi), (n))
 #else
 #define PR_CLZ(v) __builtin_clz(v)
 #define PR_UMULHI(a, b) ((uint32_t)(((uint64_t)(a) * (uint64_t)(b)) >> 32))
 #define PR_SMULHI(a, b) ((int32_t)(((int64_t)(a) * (int64_t)(b)) >> 32))
+#define PR_FUNNEL_L(lo, hi, n) ((uint32_t)(((((uint64_t)(hi) << 32) | (uint32_t)(lo)) << (n)) >> 32))
 #endif
 
 #ifdef __CUDACC__
@@ -67,7 +73,9 @@ PR_HD int64_t horner_step(int64_t acc, uint32_t t, uint64_t c)
     return hi + (int64_t)(c + PR_UMULHI((uint32_t)acc, t));
 }
 
-// a b / 2^64 for a < 2^63 + 1, b < 2^63, to within two units below
+// a b / 2^64 to within two units below, for a and b with
+// (a >> 32) (b mod 2^32) + (a mod 2^32) (b >> 32) < 2^64: both at most 2^63, or the
+// product below 2^119
 PR_HD uint64_t mulhi_near(uint64_t a, uint64_t b)
 {
     const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
@@ -75,13 +83,14 @@ PR_HD uint64_t mulhi_near(uint64_t a, uint64_t b)
     return (uint64_t)ah * bh + (mid >> 32);
 }
 
-// r 2^60 for the uniform (2 (w >> 9) + 1) 2^-24
-PR_HD uint64_t radius_fixed(uint32_t w, const NormalTables& tab)
+// r 2^(60 + shift) for the uniform (2 (w >> 9) + 1) 2^-24
+PR_HD uint64_t radius_fixed(uint32_t w, const NormalTables& tab, uint32_t& shift)
 {
     const uint32_t m = (w >> 8) | 1u;
     const uint32_t side = w >> 31;
     const uint32_t v = side ? (1u << 24) - m : m;
     const int lz = PR_CLZ(v);
+    shift = side ? (uint32_t)(lz - 5) >> 1 : (lz < 19 ? 1u : 0u);   // radius_shift(side, 31 - lz)
     const uint32_t norm = v << lz;                     // leading bit at 31
     const uint32_t t = (norm << (kSegBits + 1)) >> 1;
     const int g = (int)(((side ? 23u : 0u) + (uint32_t)(31 - lz)) << kSegBits) +
@@ -97,48 +106,52 @@ PR_HD uint64_t radius_fixed(uint32_t w, const NormalTables& tab)
     return (uint64_t)horner_step(acc, t, c01.a);
 }
 
-// |cos| 2^63, |sin| 2^63 of 2 pi u and the quarter turn, u = (2 (w >> 9) + 1) 2^-24:
-// cos(2 pi u) = (+c, -s, -c, +s)[quarter], sin(2 pi u) = (+s, +c, -s, -c)[quarter]
-PR_HD uint32_t angle_fixed(uint32_t w, const NormalTables& tab, uint64_t& c, uint64_t& s)
+// cos 2^63 and sin 2^(63 + z) of the angle 2 pi u reflected into the first eighth
+// of a turn, u = (2 (w >> 9) + 1) 2^-24; the sine's leading bit is at 62
+PR_HD void angle_fixed(uint32_t w, const NormalTables& tab, uint64_t& c, uint64_t& s, uint32_t& z)
 {
-    const U64x2 node = tab.nodes[(w >> 20) & 1023u];
-    const uint32_t n = ((w >> 8) & 4095u) | 1u;        // b = n 2 pi 2^-24
-    const uint32_t n2 = n * n, n2s = n2 << 8;
-    const uint32_t k3 = (uint32_t)kSin3 - (PR_UMULHI(n2s, (uint32_t)kSin5) >> 16);
-    const uint64_t k1 = kSin1 - PR_UMULHI(n2s, k3);    // sin(b) / n, 2^-73 units
-    const uint64_t sb = (((uint64_t)((uint32_t)(k1 >> 32) * n) << 32) + (uint64_t)(uint32_t)k1 * n) >> 9;
+    const uint32_t x = (w >> 8) ^ (uint32_t)((int32_t)(w << 2) >> 31);   // odd eighths run backwards
+    const U64x2 node = tab.nodes[(x >> 11) & 1023u];   // cos 2^63, sin 2^64
+    const uint32_t n = (x & 2047u) | 1u;               // b = n d, d = 2 pi 2^-24
+    const uint32_t n2 = n * n, n2s = n2 << 10;
+    const uint32_t k3 = (uint32_t)kSin3 - ((PR_UMULHI(n2s, (uint32_t)kSin5) + (1u << 23)) >> 24);
+    const uint64_t k1 = kSin1 - (((uint64_t)n2s * k3) >> 24);   // sin(b) / n, 2^-84 units
     const uint64_t k2 = kCos2 - PR_UMULHI(n2s, (uint32_t)kCos4);   // (1 - cos b) / n^2, 2^-97 units
-    const uint64_t e = ((uint64_t)(uint32_t)(k2 >> 32) * n2 + PR_UMULHI((uint32_t)k2, n2)) >> 1;
-    c = node.a - mulhi_near(node.a, e) - mulhi_near(node.b, sb);
-    s = node.b - mulhi_near(node.b, e) + mulhi_near(node.a, sb);
-    return w >> 30;
+    const uint64_t e = (uint64_t)(uint32_t)(k2 >> 32) * n2s + PR_UMULHI((uint32_t)k2, n2s);   // 1 - cos b, 2^-75 units
+    const uint64_t sb = (uint64_t)(uint32_t)(k1 >> 32) * (n << 12) + PR_UMULHI((uint32_t)k1, n << 12);   // sin b, 2^-64
+    c = node.a - (mulhi_near(node.a, e) >> 11) - (mulhi_near(node.b, sb) >> 1);
+    // sin(node) - sin(node) (1 - cos b) + (cos(node) sin(b) / n) n in 2^-96 units
+    const uint64_t k = mulhi_near(node.a, k1), f = mulhi_near(node.b, e);   // 2^-83 and 2^-75 units
+    const int64_t low = (int64_t)((uint64_t)(uint32_t)k * (n << 13)) - (int64_t)((uint64_t)(uint32_t)f << 21);
+    const uint64_t high = node.b + (uint64_t)(uint32_t)(k >> 32) * (n << 13) - ((f >> 32) << 21) + (uint64_t)(low >> 32);
+    const uint32_t s2 = (uint32_t)(high >> 32), s1 = (uint32_t)high, s0 = (uint32_t)low;
+    z = (uint32_t)PR_CLZ((int)s2);                     // (sin > 2^-21.4: s2 is not 0)
+    s = (((uint64_t)PR_FUNNEL_L(s1, s2, z) << 32) | PR_FUNNEL_L(s0, s1, z)) >> 1;
 }
 
-// The encoding of v 2^-59 (v > 0) rounded to nearest, ties up; `sign` in bit 31
-PR_HD uint64_t encode_2m59(uint64_t v, uint32_t sign)
+// The encoding of v 2^-(59 + shift) rounded to nearest, ties up (2^32 <= v < 2^63)
+PR_HD uint64_t encode_2m59(uint64_t v, uint32_t shift)
 {
-    uint32_t hi = (uint32_t)(v >> 32);
-    int lz = 0;
-    if (hi == 0u) {   // below 2^-27: rare
-        v <<= 32;
-        hi = (uint32_t)(v >> 32);
-        lz = 32;
-    }
-    const int z = PR_CLZ(hi | 1u);
+    const int z = PR_CLZ((int)(uint32_t)(v >> 32));
     v <<= z;
     const uint64_t bits = (v >> 11) + ((v >> 10) & 1u);
-    return bits + ((uint64_t)(((uint32_t)(1026 - lz - z) << 20) | sign) << 32);
+    return bits + ((uint64_t)((1026u - shift - (uint32_t)z) << 20) << 32);
 }
 
-// The normals z0 = r cos, z1 = r sin of the words w0 (radius) and w1 (angle).
+// The normals z0 = r cos, z1 = r sin of the words w0 (radius) and w1 (angle):
+// the reflected pair changes places in the odd eighths of a turn, the signs
+// are those of the quarter.
 PR_HD void box_muller_fixed(uint32_t w0, uint32_t w1, const NormalTables& tab, uint64_t& z0, uint64_t& z1)
 {
-    const uint64_t r = radius_fixed(w0, tab);
+    uint32_t shift, z;
+    const uint64_t r = radius_fixed(w0, tab, shift);
     uint64_t c, s;
-    const uint32_t q = angle_fixed(w1, tab, c, s);
-    const uint64_t a = mulhi_near(r, q & 1u ? s : c), b = mulhi_near(r, q & 1u ? c : s);
-    z0 = encode_2m59(a, ((q + 1u) & 2u) << 30);
-    z1 = encode_2m59(b, (q & 2u) << 30);
+    angle_fixed(w1, tab, c, s, z);
+    const uint64_t a = encode_2m59(mulhi_near(r, c), shift), b = encode_2m59(mulhi_near(r, s), shift + z);
+    const uint32_t q = w1 >> 30;
+    const bool swap = ((w1 >> 30) ^ (w1 >> 29)) & 1u;
+    z0 = (swap ? b : a) | ((uint64_t)(((q + 1u) & 2u) << 30) << 32);
+    z1 = (swap ? a : b) | ((uint64_t)((q & 2u) << 30) << 32);
 }
 
 }  // namespace pr

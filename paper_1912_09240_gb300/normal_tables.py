@@ -2,16 +2,19 @@
 
 The binary64 kernels take their Box-Muller normals r cos(theta), r sin(theta)
 from integer arithmetic (csrc/normal64.cuh): the radius r(u) = sqrt(-2 ln u)
-from piecewise polynomials, the angle from cosines and sines at equidistant
-nodes and the angle-addition formulas.  Everything here is computed with
-``decimal`` and integers, so the header is the same on every machine.
+from piecewise polynomials, the angle, reflected into an eighth of a turn, from
+cosines and sines at equidistant nodes and the angle-addition formulas.
+Everything here is computed with ``decimal`` and integers, so the header is the
+same on every machine.
 
 Radius: u = M 2^-24 with M an odd 24-bit integer.  For M < 2^23 the variable
 is M, otherwise 2^24 - M (r is smooth in the logarithm of both; near u = 1 it
 behaves like sqrt(2 (1 - u))).  Each binade 2^e <= M' < 2^(e+1) is cut into 32
 equal segments, and on each r is the polynomial of degree 7 through its
-Chebyshev points (error below 2^-60), as coefficients in sigma = tau / 2,
-tau in [0, 1) the place in the segment.
+Chebyshev points (relative error below 2^-60), as coefficients in sigma = tau / 2,
+tau in [0, 1) the place in the segment, in units of 2^-(60 + shift): the shift of
+the binade (``radius_shift``) puts r between 2^61 and 2^63 units, so that a small
+radius keeps as many bits as a large one.
 """
 from __future__ import annotations
 
@@ -22,8 +25,8 @@ D = decimal.Decimal
 SEG_BITS = 5
 DEGREE = 7
 BINADES = 23
-TAIL_SHIFT = 6        # c5..c7 are kept in units of 2^(TAIL_SHIFT - 60)
-NODE_BITS = 10        # nodes per quarter turn: 2^10
+TAIL_SHIFT = 8        # c5..c7 are kept in units of 2^(TAIL_SHIFT - 60 - shift)
+NODE_BITS = 10        # nodes per eighth of a turn: 2^10
 
 
 def _pi(prec: int) -> D:
@@ -75,8 +78,13 @@ def _rint(v: D) -> int:
     return int(v.to_integral_value(rounding=decimal.ROUND_HALF_EVEN))
 
 
+def radius_shift(side: int, e: int) -> int:
+    """r 2^(60 + shift) is at least 2^61 and below 2^63 on the binade 2^e of u (side 0) or 1 - u (side 1)."""
+    return (26 - e) >> 1 if side else int(e >= 13)
+
+
 def radius_table():
-    """[segment][DEGREE + 1] integers: c_k 2^k 2^60 (k <= 4), the rest in units of 2^(TAIL_SHIFT - 60)."""
+    """[segment][DEGREE + 1] integers: c_k 2^k 2^(60 + shift) (k <= 4), the rest in units of 2^(TAIL_SHIFT - 60 - shift)."""
     n = DEGREE + 1
     pts, rows = _chebyshev(n)
     out = []
@@ -89,15 +97,17 @@ def radius_table():
                     m = D(2) ** (e - 24) * (1 + (g + p) / segs)   # u or 1 - u
                     vals.append((-2 * (1 - m if side else m).ln()).sqrt())
                 coef = [sum(rows[k][i] * vals[k] for k in range(n)) for i in range(n)]
-                scaled = [c * 2 ** (60 + i - (TAIL_SHIFT if i > 4 else 0)) for i, c in enumerate(coef)]
+                one = 60 + radius_shift(side, e)
+                assert all(2 ** 60 < v * 2 ** one < 2 ** 63 for v in vals)
+                scaled = [c * 2 ** (one + i - (TAIL_SHIFT if i > 4 else 0)) for i, c in enumerate(coef)]
                 out.append([_rint(c) for c in scaled])
     return out
 
 
 def node_table():
-    """[node](cos, sin) 2^63 of node pi/2 / 2^NODE_BITS."""
+    """[node](cos 2^63, sin 2^64) of node pi/4 / 2^NODE_BITS."""
     pi = _pi(40)
-    return [tuple(_rint(v * 2 ** 63) for v in _cos_sin(pi / 2 * i / (1 << NODE_BITS)))
+    return [tuple(_rint(v * 2 ** k) for v, k in zip(_cos_sin(pi / 4 * i / (1 << NODE_BITS)), (63, 64)))
             for i in range(1 << NODE_BITS)]
 
 
@@ -107,9 +117,9 @@ def header() -> str:
         rad, nodes = radius_table(), node_table()
         d = 2 * _pi(40) / 2 ** 24                      # the angle of one unit
         consts = {
-            "kSin1": _rint(d * 2 ** 73), "kSin3": _rint(d ** 3 / 6 * 2 ** 97),
-            "kSin5": _rint(d ** 5 / 120 * 2 ** 137),
-            "kCos2": _rint(d ** 2 / 2 * 2 ** 97), "kCos4": _rint(d ** 4 / 24 * 2 ** 121),
+            "kSin1": _rint(d * 2 ** 84), "kSin3": _rint(d ** 3 / 6 * 2 ** 98),
+            "kSin5": _rint(d ** 5 / 120 * 2 ** 144),
+            "kCos2": _rint(d ** 2 / 2 * 2 ** 97), "kCos4": _rint(d ** 4 / 24 * 2 ** 119),
         }
     for c in rad:
         assert all(abs(v) < 2 ** 63 for v in c[:5]) and all(abs(v) < 2 ** 31 for v in c[5:])

@@ -67,6 +67,44 @@ def test_normals_against_long_double(tmp_path, kind):
         assert np.all(err <= 2.0 ** -56 + 0.5 * np.spacing(np.abs(got)) * 1.001)
 
 
+def _all_words(kind):
+    """Every radius with one angle, or every angle with one radius (of which the words' upper 23 bits count)."""
+    k = (np.arange(1 << 23, dtype=np.uint64) << 9).astype(np.uint32)
+    one = np.full(k.size, {"angles": 0x12345600, "angles, u near 1": 0xFFFFFE00, "radii": 0x02345600}[kind], np.uint32)
+    return (k, one) if kind == "radii" else (one, k)
+
+
+@pytest.mark.parametrize("kind", ["angles", "angles, u near 1", "radii"])
+def test_relative_error_at_every_size(tmp_path, kind):
+    """The error relative to the normal, however small it is: half an ulp of the rounding (2^-53 at most)
+    and the fixed-point pair's, whose worst part is the sine's: from the first node on (sin > 2^-10.4) its
+    entry is rounded to 2^-65, 2^-54.6 at most; at node 0 it is n times a series, off by a unit of 2^31.4
+    in a term of 2^-23.3, 2^-54.7; radius, cosine and product are below 2^-58 each.  2^-54 covers the sum."""
+    if np.finfo(np.longdouble).eps > 2.0 ** -63:
+        pytest.skip("long double is binary64 here")
+    normal_tables.write(str(tmp_path / "normal_tables.h"))
+    (tmp_path / "n.cpp").write_text(SRC)
+    so = str(tmp_path / "n.so")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", str(tmp_path), "-I", b.CSRC, "-o", so,
+                           str(tmp_path / "n.cpp")])
+    w0, w1 = _all_words(kind)
+    z = np.empty((2, w0.size))
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    ctypes.CDLL(so).normals(p(w0), p(w1), ctypes.c_long(w0.size), p(z[0]), p(z[1]))
+    two24 = np.longdouble(1 << 24)
+    for lo in range(0, w0.size, 1 << 20):     # in parts: long doubles take 16 bytes each
+        part = slice(lo, lo + (1 << 20))
+        m = (2 * (w0[part] >> 9).astype(np.int64) + 1)
+        r = np.sqrt(-2 * np.where(m > (1 << 23), np.log1p(-(two24 - m) / two24), np.log(m / two24)))
+        a = (2 * (w1[part] >> 9).astype(np.int64) + 1)
+        q = (a + (1 << 21)) >> 22
+        x = (a - (q << 22)).astype(np.longdouble) * (np.longdouble(2) * np.arccos(np.longdouble(-1)) / two24)
+        c, s = np.cos(x), np.sin(x)
+        for got, want in ((z[0, part], r * np.choose(q & 3, [c, -s, -c, s])),
+                          (z[1, part], r * np.choose(q & 3, [s, c, -s, -c]))):
+            assert np.all(np.abs(got.astype(np.longdouble) - want) <= (2.0 ** -53 + 2.0 ** -54) * np.abs(want))
+
+
 def _step(bins, match, d, n, steps, eps=0.1, x0=None, y0=None):
     import torch
     from paper_1912_09240_gb300 import _lib as L
