@@ -435,13 +435,10 @@ extern "C" pr_status pr_coarse_create(const pr_model* model, const pr_grid* grid
         if (scratch) cudaFree(scratch);
         return rc;
     };
-    // one allocation up to 1024 bins (the scratch then stays with the handle:
-    // an allocation and its release cost about as much as a squaring)
-    const size_t extra = (nn + 3 * (size_t)I + 1) * 8;
-    const bool one = I <= 1024;
-    if (cudaMalloc(&P, nn * 8 + (one ? extra : 0)) != cudaSuccess) return fail(PR_ERR_NOMEM);
-    if (!one && cudaMalloc(&scratch, extra) != cudaSuccess) return fail(PR_ERR_NOMEM);
-    double* W = one ? P + nn : scratch;
+    // (an allocation of its own, released again: a handle holds its matrix alone)
+    if (cudaMalloc(&P, nn * 8) != cudaSuccess || cudaMalloc(&scratch, (nn + 3 * (size_t)I + 1) * 8) != cudaSuccess)
+        return fail(PR_ERR_NOMEM);
+    double* W = scratch;
     double *sub = W + nn, *dia = sub + I, *sup = dia + I, *ybar_dev = sup + I;
     const GridDev g = make_grid(*grid);
     if (chem) {   // ybar first; it must be positive and finite
@@ -480,7 +477,7 @@ extern "C" pr_status pr_coarse_create(const pr_model* model, const pr_grid* grid
         band = std::min(2 * band, I);
     }
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return fail(PR_ERR_CUDA);
-    if (scratch) cudaFree(scratch);
+    cudaFree(scratch);
     auto* h = new CoarseHandle;
     h->g = g;
     h->P = P;

@@ -26,3 +26,21 @@ def test_propagator_matches_oracle(bins, kind, dT):
     want = oracle.coarse_propagator(oracle.Model(kind, 1, **par), oracle.Grid(bins, -3.0, 2.5), dT)
     # the bound of the other propagator tests: both exponentials within 1e-12
     assert np.max(np.abs(P.cpu().numpy() - want)) <= 1e-12
+
+
+@pytest.mark.parametrize("bins", [700, 1024])
+def test_a_handle_holds_its_matrix_alone(bins):
+    """Device memory of eight handles: the matrix each, rounded up to the allocator's 2 MiB."""
+    import torch
+    from paper_1912_09240_gb300 import _lib as L
+    b.build()
+    make = lambda: L.pr_coarse_create(L.Model(L.PR_MODEL_OU, 1, 0.5, 1.5, 0.7), L.Grid(bins, -3.0, 2.5), 0.1)
+    L.pr_coarse_destroy(make())
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    handles = [make() for _ in range(8)]
+    torch.cuda.synchronize()
+    held = before - torch.cuda.mem_get_info()[0]
+    for h in handles:
+        L.pr_coarse_destroy(h)
+    assert held <= 8 * (8 * bins * bins + (2 << 20))
