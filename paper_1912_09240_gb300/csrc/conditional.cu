@@ -496,8 +496,10 @@ constexpr int kSelPer = 8;
 constexpr int kSelOut = kSelThreads * kSelPer;   // consecutive outputs per CTA
 static_assert(kSelPer % 4 == 0, "a thread's outputs start on a Philox block of the strata draws");
 // Cumulative weights staged per CTA: the particles of kSelOut outputs are about
-// as many (19 % more are held; the rest of a longer range is read from global
-// memory).  With 2432 of them eight CTAs fit an SM, with 4096 five.
+// as many (19 % more are held; of a longer range every k-th).  With 2432 of them
+// eight CTAs fit an SM, with 4096 five.  pr_resample of 9 x 2^20 outputs: even
+// weights 129 us (141 with 4096), lognormal ones with a coefficient of variation
+// of 7 142 (160), of 90 148 (170; 194 with the rest of the range in global memory).
 constexpr int kSelStage = 2432;
 
 // The particles of the first and last output of every selection CTA: one
@@ -533,33 +535,66 @@ select_bounds_kernel(const uint64_t* __restrict__ C, const uint64_t* __restrict_
     *out = first_above(C + (int64_t)s * n, p0, p1, u);
 }
 
-// Searches over cumulative weights given by an accessor v (index -> C):
-// the smallest index in [a, b] with C > u, given C_b > u; and the same from a
-// known lower bound a, in steps 1, 2, 4, .. and then a search of the last
-// step (C_hi > u).
-template <typename V, typename Idx>
-__device__ __forceinline__ Idx sel_search(const V& v, Idx a, Idx b, uint64_t u)
+// Searches over increasing cumulative weights: the smallest index in [a, b] with
+// C > u, given C_b > u; and the same from a known lower bound a, in steps
+// 1, 2, 4, .. and then a search of the last step (C_hi > u).
+template <typename Idx>
+__device__ __forceinline__ Idx sel_search(const uint64_t* C, Idx a, Idx b, uint64_t u)
 {
     while (a < b) {
-        const Idx mid = (a + b) >> 1;
-        if (v(mid) > u) b = mid; else a = mid + 1;
+        const Idx mid = a + ((b - a) >> 1);
+        if (C[mid] > u) b = mid; else a = mid + 1;
     }
     return a;
 }
 
-template <typename V, typename Idx>
-__device__ __forceinline__ Idx sel_gallop(const V& v, Idx a, Idx hi, uint64_t u)
+__device__ __forceinline__ int sel_gallop(const uint64_t* C, int a, int hi, uint64_t u)
 {
-    if (v(a) > u) return a;
-    Idx step = 1;
+    if (C[a] > u) return a;
+    int step = 1;
     for (;;) {                          // C_a <= u < C_hi, so a < hi
-        const Idx nx = a + step;
-        if (nx >= hi) return sel_search(v, a + 1, hi, u);
-        if (v(nx) > u) return sel_search(v, a + 1, nx, u);
+        const int nx = a + step;
+        if (nx >= hi) return sel_search(C, a + 1, hi, u);
+        if (C[nx] > u) return sel_search(C, a + 1, nx, u);
         a = nx;
         step <<= 1;
     }
 }
+
+// The particle of each of a thread's increasing strata points, relative to the
+// CTA's first.  SelStaged: the whole range's cumulative weights in shared memory.
+struct SelStaged {
+    const uint64_t* cs;
+    int hi, p = 0;
+    __device__ __forceinline__ uint32_t first(uint64_t u) { return (uint32_t)(p = sel_search(cs, 0, hi, u)); }
+    __device__ __forceinline__ uint32_t next(uint64_t u) { return (uint32_t)(p = sel_gallop(cs, p, hi, u)); }
+};
+
+// SelStrided: a longer range (uneven weights), the last of every `stride`
+// cumulative weights in shared memory: they lead to the `stride` particles
+// that are then searched in global memory.
+struct SelStrided {
+    const uint64_t *cs, *C;
+    int m;              // staged
+    uint32_t stride, hi;
+    int k = 0;
+    uint32_t p = 0;
+    __device__ __forceinline__ uint32_t within(uint64_t u)
+    {
+        const uint32_t a = (uint32_t)k * stride;
+        return p = sel_search(C, a > p ? a : p, hi - a < stride ? hi : a + (stride - 1u), u);
+    }
+    __device__ __forceinline__ uint32_t first(uint64_t u)
+    {
+        k = sel_search(cs, 0, m - 1, u);
+        return within(u);
+    }
+    __device__ __forceinline__ uint32_t next(uint64_t u)
+    {
+        k = sel_gallop(cs, k, m - 1, u);
+        return within(u);
+    }
+};
 
 __device__ __forceinline__ int sel_pad(int i) { return i + (i >> 5); }
 
@@ -567,10 +602,9 @@ __device__ __forceinline__ int sel_pad(int i) { return i + (i >> 5); }
 // kSelPer, so they take whole Philox blocks of four draws): their strata
 // points first (independent blocks, all in flight), then a search for the
 // first particle and a gallop from the previous one for the rest; the
-// particles, relative to `base`, go to sp.
-template <typename V, typename Idx>
-__device__ __forceinline__ void select_run(const V& v, Idx base, Idx hi, const StrataPoint& U, uint32_t j0,
-                                           int jj0, int cnt, uint32_t* sp)
+// particles go to sp.
+template <typename F>
+__device__ __forceinline__ void select_run(F find, const StrataPoint& U, uint32_t j0, int jj0, int cnt, uint32_t* sp)
 {
     const uint32_t j = j0 + (uint32_t)jj0;
     uint32_t q2, r2;
@@ -608,15 +642,10 @@ __device__ __forceinline__ void select_run(const V& v, Idx base, Idx hi, const S
         }
     }
     const int m = min(kSelPer, cnt - jj0);
-    Idx p = sel_search(v, base, hi, u[0]);
-    sp[sel_pad(jj0)] = (uint32_t)(p - base);
+    sp[sel_pad(jj0)] = find.first(u[0]);
 #pragma unroll
-    for (int k = 1; k < kSelPer; ++k) {
-        if (k < m) {
-            p = sel_gallop(v, p, hi, u[k]);
-            sp[sel_pad(jj0 + k)] = (uint32_t)(p - base);
-        }
-    }
+    for (int k = 1; k < kSelPer; ++k)
+        if (k < m) sp[sel_pad(jj0 + k)] = find.next(u[k]);
 }
 
 // Copies dst[k kSelThreads] = src[pr[k]] for the kSelPer outputs of this
@@ -637,7 +666,7 @@ __device__ __forceinline__ void gather_rows(const T* __restrict__ src, T* __rest
 // One CTA takes kSelOut consecutive outputs, whose particles lie between
 // those of its first and last output (U and C both increase).  Their
 // cumulative weights are staged in shared memory (up to kSelStage of them;
-// beyond, they are read from global memory).  Each thread finds the particles
+// beyond, an even sample of them).  Each thread finds the particles
 // of kSelPer consecutive outputs into shared memory; the indices and the
 // gathered states are then written with consecutive outputs on consecutive
 // threads.
@@ -664,24 +693,24 @@ select_gather_kernel(const uint64_t* __restrict__ C, const uint64_t* __restrict_
         const int64_t* bd = bounds + ((int64_t)s * gridDim.x + blockIdx.x) * 2;
         lo = bd[0];
         const int64_t hi = bd[1];
-        const uint64_t* Cs = C + (int64_t)s * n;
-        const int64_t span = hi - lo + 1;
-        const int m = (int)min(span, (int64_t)kSelStage);
+        const uint64_t* Cs = C + (int64_t)s * n + lo;
+        const uint32_t last = (uint32_t)(hi - lo);           // (below 2^32: p < n)
+        const uint32_t stride = last / kSelStage + 1u;
+        const int m = (int)(last / stride) + 1;
         if (threadIdx.x == 0) s_Q = Tw / (uint64_t)n;
-        for (int k = threadIdx.x; k < m; k += kSelThreads) cs[k] = Cs[lo + k];
+        if (stride == 1u)
+            for (int k = threadIdx.x; k < m; k += kSelThreads) cs[k] = Cs[k];
+        else
+            for (int k = threadIdx.x; k < m; k += kSelThreads)
+                cs[k] = Cs[last - (uint32_t)k * stride < stride ? last : (uint32_t)k * stride + (stride - 1u)];
         __syncthreads();
         const uint64_t Q = s_Q;
         const StrataPoint U = make_strata(Q, (uint32_t)(Tw - Q * (uint64_t)n), n, mode, k0, k1, chi,
                                           slice0 + (uint32_t)s);
         const int jj0 = threadIdx.x * kSelPer;
         if (jj0 < cnt) {
-            if (span <= kSelStage) {        // the whole range staged: 32-bit indices into it
-                const auto v = [&](int i) { return cs[i]; };
-                select_run(v, 0, (int)span - 1, U, (uint32_t)j0, jj0, cnt, sp);
-            } else {
-                const auto v = [&](int64_t p) { return p - lo < m ? cs[p - lo] : Cs[p]; };
-                select_run(v, lo, hi, U, (uint32_t)j0, jj0, cnt, sp);
-            }
+            if (stride == 1u) select_run(SelStaged{cs, m - 1}, U, (uint32_t)j0, jj0, cnt, sp);
+            else select_run(SelStrided{cs, Cs, m, stride, last}, U, (uint32_t)j0, jj0, cnt, sp);
         }
     } else {
         for (int jj = threadIdx.x; jj < cnt; jj += kSelThreads) sp[sel_pad(jj)] = (uint32_t)jj;

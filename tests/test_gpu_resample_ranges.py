@@ -44,3 +44,29 @@ def test_indices_and_weighted_cdf(kind, n, mode):
     L.pr_restrict_weighted(L.PR_F32, gx, False, gw, n, 2, L.Grid(100, -3.0, 3.0), cdf, wr)
     np.testing.assert_array_equal(cdf.cpu().numpy(),
                                   oracle.restrict_weighted(x.astype(np.float64), w, oracle.Grid(100, -3.0, 3.0)))
+
+
+@pytest.mark.parametrize("kind", ["sorted", "runs", "one"])
+@pytest.mark.parametrize("n", [4866, 9730, 300007])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_ranges_longer_than_the_staged_one(kind, n, mode):
+    """A CTA's outputs spread over up to all particles: ascending weights of five decades, zero weights
+    but for short runs, and one particle that holds nearly all; the ranges of the smaller sizes are just
+    above one, two and four times the staged one."""
+    import torch
+    from paper_1912_09240_gb300 import _lib as L
+    b.build()
+    r = np.random.default_rng(n)
+    w = {"sorted": lambda: np.sort(np.exp(2.5 * r.normal(0, 1, n))),
+         "runs": lambda: ((np.arange(n) % 1000) < 3) * r.random(n) + (np.arange(n) == n - 1),
+         "one": lambda: np.where(np.arange(n) == n // 3, 1e6, 1e-3 * r.random(n))}[kind]()
+    w = np.stack([w / w.sum(), (w / w.sum())[::-1]])
+    x = r.normal(0, 1, (2, n))
+    gw, gx = torch.tensor(w.copy(), device="cuda"), torch.tensor(x, device="cuda")
+    idx = torch.empty(2, n, dtype=torch.int32, device="cuda")
+    xo = torch.empty_like(gx)
+    ws = torch.empty(L.pr_resample_workspace(n, 2), dtype=torch.uint8, device="cuda")
+    L.pr_resample(L.PR_F64, 1, gx, None, False, gw, n, 2, 3, mode, L.Rng(5, 9), idx, xo, None, ws)
+    want = oracle.resample(w, mode, 5, 3, problem=9)
+    np.testing.assert_array_equal(idx.cpu().numpy().view(np.uint32), want)
+    np.testing.assert_array_equal(xo.cpu().numpy(), np.take_along_axis(x, want.astype(np.int64), 1))
