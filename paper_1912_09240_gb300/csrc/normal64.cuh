@@ -12,12 +12,12 @@
 //           binade;
 //   angle   2 pi u1 reflected into an eighth of a turn = node + b: cos and sin of
 //           the 1024 nodes, of b < 2^-10.3 from its series, and the addition
-//           formulas.  The sine is a sum of positive terms there, kept in 96 bits
-//           and normalised to 63, so that it keeps its bits where it is small.
-// So the normals have the same relative error at every size, before the one
-// rounding to binary64 2^-59.3 rms and 2^-54.6 at most (at the first nodes, whose
-// sines are rounded to 2^-65), after it 2^-54.2 rms; a pair in absolute fixed
-// point lost its bits where it is small (2^-47.5 rms, 2^-41 below 2^-12).
+//           formulas.  The sine is a sum of positive terms there; its terms are
+//           scaled by 2^z, z the leading zeros of the angle, so that it keeps
+//           its bits where it is small.
+// So the normals have the same relative error at every size: before the one
+// rounding to binary64 2^-58.6 rms and 2^-55.3 at most, after it 2^-54.2 rms (in
+// absolute fixed point a small normal loses bits: 2^-47.5 rms, 2^-41 below 2^-12).
 // Tables and constants: normal_tables.py (the header it writes is included by
 // the translation unit that holds the tables).
 #pragma once
@@ -28,12 +28,10 @@
 #define PR_CLZ(v) __clz((int)(v))
 #define PR_UMULHI(a, b) __umulhi((a), (b))
 #define PR_SMULHI(a, b) __mulhi((a), (b))
-#define PR_FUNNEL_L(lo, hi, n) __funnelshift_l((lo), (hi), (n))
 #else
 #define PR_CLZ(v) __builtin_clz(v)
 #define PR_UMULHI(a, b) ((uint32_t)(((uint64_t)(a) * (uint64_t)(b)) >> 32))
 #define PR_SMULHI(a, b) ((int32_t)(((int64_t)(a) * (int64_t)(b)) >> 32))
-#define PR_FUNNEL_L(lo, hi, n) ((uint32_t)(((((uint64_t)(hi) << 32) | (uint32_t)(lo)) << (n)) >> 32))
 #endif
 
 #ifdef __CUDACC__
@@ -53,7 +51,7 @@ struct alignas(16) U64x2 {
 // The tables, 16-byte aligned, in the order the header holds them.
 struct NormalTables {
     const U64x2* radius;   // [kRadiusSegments][3]
-    const U64x2* nodes;    // [kNodes] (cos, sin)
+    const U64x2* nodes;    // [kNodes] (cos 2^63, sin 2^(62 + z))
     const int32_t* c7;     // [kRadiusSegments]
 };
 
@@ -73,9 +71,7 @@ PR_HD int64_t horner_step(int64_t acc, uint32_t t, uint64_t c)
     return hi + (int64_t)(c + PR_UMULHI((uint32_t)acc, t));
 }
 
-// a b / 2^64 to within two units below, for a and b with
-// (a >> 32) (b mod 2^32) + (a mod 2^32) (b >> 32) < 2^64: both at most 2^63, or the
-// product below 2^119
+// a b / 2^64 for a < 2^63, b <= 2^63, to within two units below
 PR_HD uint64_t mulhi_near(uint64_t a, uint64_t b)
 {
     const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
@@ -106,27 +102,24 @@ PR_HD uint64_t radius_fixed(uint32_t w, const NormalTables& tab, uint32_t& shift
     return (uint64_t)horner_step(acc, t, c01.a);
 }
 
-// cos 2^63 and sin 2^(63 + z) of the angle 2 pi u reflected into the first eighth
-// of a turn, u = (2 (w >> 9) + 1) 2^-24; the sine's leading bit is at 62
+// cos 2^63 and sin 2^(62 + z) of the angle 2 pi u reflected into the first eighth
+// of a turn, u = (2 (w >> 9) + 1) 2^-24; z such that the sine is between 2^60.4 and
+// 2^61.7
 PR_HD void angle_fixed(uint32_t w, const NormalTables& tab, uint64_t& c, uint64_t& s, uint32_t& z)
 {
     const uint32_t x = (w >> 8) ^ (uint32_t)((int32_t)(w << 2) >> 31);   // odd eighths run backwards
-    const U64x2 node = tab.nodes[(x >> 11) & 1023u];   // cos 2^63, sin 2^64
+    const U64x2 node = tab.nodes[(x >> 11) & 1023u];
     const uint32_t n = (x & 2047u) | 1u;               // b = n d, d = 2 pi 2^-24
+    z = (uint32_t)PR_CLZ((int)((x << 11) | 2048u));    // (the sine is 0.90 to 1 times its angle)
     const uint32_t n2 = n * n, n2s = n2 << 10;
     const uint32_t k3 = (uint32_t)kSin3 - ((PR_UMULHI(n2s, (uint32_t)kSin5) + (1u << 23)) >> 24);
     const uint64_t k1 = kSin1 - (((uint64_t)n2s * k3) >> 24);   // sin(b) / n, 2^-84 units
     const uint64_t k2 = kCos2 - PR_UMULHI(n2s, (uint32_t)kCos4);   // (1 - cos b) / n^2, 2^-97 units
-    const uint64_t e = (uint64_t)(uint32_t)(k2 >> 32) * n2s + PR_UMULHI((uint32_t)k2, n2s);   // 1 - cos b, 2^-75 units
-    const uint64_t sb = (uint64_t)(uint32_t)(k1 >> 32) * (n << 12) + PR_UMULHI((uint32_t)k1, n << 12);   // sin b, 2^-64
-    c = node.a - (mulhi_near(node.a, e) >> 11) - (mulhi_near(node.b, sb) >> 1);
-    // sin(node) - sin(node) (1 - cos b) + (cos(node) sin(b) / n) n in 2^-96 units
-    const uint64_t k = mulhi_near(node.a, k1), f = mulhi_near(node.b, e);   // 2^-83 and 2^-75 units
-    const int64_t low = (int64_t)((uint64_t)(uint32_t)k * (n << 13)) - (int64_t)((uint64_t)(uint32_t)f << 21);
-    const uint64_t high = node.b + (uint64_t)(uint32_t)(k >> 32) * (n << 13) - ((f >> 32) << 21) + (uint64_t)(low >> 32);
-    const uint32_t s2 = (uint32_t)(high >> 32), s1 = (uint32_t)high, s0 = (uint32_t)low;
-    z = (uint32_t)PR_CLZ((int)s2);                     // (sin > 2^-21.4: s2 is not 0)
-    s = (((uint64_t)PR_FUNNEL_L(s1, s2, z) << 32) | PR_FUNNEL_L(s0, s1, z)) >> 1;
+    const uint64_t e = ((uint64_t)(uint32_t)(k2 >> 32) * n2 + PR_UMULHI((uint32_t)k2, n2)) >> 1;   // 1 - cos b, 2^-64
+    const uint32_t nz = n << (z + 11u);                // (n below 2^11, and 2^(21 - z) at node 0)
+    const uint64_t sb = (uint64_t)(uint32_t)(k1 >> 32) * nz + PR_UMULHI((uint32_t)k1, nz);   // sin b, 2^-(63 + z)
+    c = node.a - mulhi_near(node.a, e) - ((mulhi_near(node.b, sb) >> (2u * z)) << 2);
+    s = node.b - mulhi_near(node.b, e) + mulhi_near(node.a, sb);
 }
 
 // The encoding of v 2^-(59 + shift) rounded to nearest, ties up (2^32 <= v < 2^63)
@@ -147,7 +140,7 @@ PR_HD void box_muller_fixed(uint32_t w0, uint32_t w1, const NormalTables& tab, u
     const uint64_t r = radius_fixed(w0, tab, shift);
     uint64_t c, s;
     angle_fixed(w1, tab, c, s, z);
-    const uint64_t a = encode_2m59(mulhi_near(r, c), shift), b = encode_2m59(mulhi_near(r, s), shift + z);
+    const uint64_t a = encode_2m59(mulhi_near(r, c), shift), b = encode_2m59(mulhi_near(r, s), shift + z - 1u);
     const uint32_t q = w1 >> 30;
     const bool swap = ((w1 >> 30) ^ (w1 >> 29)) & 1u;
     z0 = (swap ? b : a) | ((uint64_t)(((q + 1u) & 2u) << 30) << 32);

@@ -105,9 +105,11 @@ def radius_table():
 
 
 def node_table():
-    """[node](cos 2^63, sin 2^64) of node pi/4 / 2^NODE_BITS."""
+    """[node](cos 2^63, sin 2^(62 + z)) of node pi/4 / 2^NODE_BITS, z the zeros in front of its number in
+    NODE_BITS bits: an angle between this node and the next has them in front of it too."""
     pi = _pi(40)
-    return [tuple(_rint(v * 2 ** k) for v, k in zip(_cos_sin(pi / 4 * i / (1 << NODE_BITS)), (63, 64)))
+    return [tuple(_rint(v * 2 ** k) for v, k in zip(_cos_sin(pi / 4 * i / (1 << NODE_BITS)),
+                                                    (63, 62 + NODE_BITS - i.bit_length())))
             for i in range(1 << NODE_BITS)]
 
 

@@ -77,9 +77,9 @@ def _all_words(kind):
 @pytest.mark.parametrize("kind", ["angles", "angles, u near 1", "radii"])
 def test_relative_error_at_every_size(tmp_path, kind):
     """The error relative to the normal, however small it is: half an ulp of the rounding (2^-53 at most)
-    and the fixed-point pair's, whose worst part is the sine's: from the first node on (sin > 2^-10.4) its
-    entry is rounded to 2^-65, 2^-54.6 at most; at node 0 it is n times a series, off by a unit of 2^31.4
-    in a term of 2^-23.3, 2^-54.7; radius, cosine and product are below 2^-58 each.  2^-54 covers the sum."""
+    and the fixed-point pair's: the sine at node 0, n times a series that is off by a unit of 2^31.4 in a
+    term of 2^-23.3, 2^-54.7; the product of radius and sine, two units of 2^57.6, 2^-56.6; radius, cosine
+    and the other nodes' sines below 2^-58 each.  2^-54 covers the sum."""
     if np.finfo(np.longdouble).eps > 2.0 ** -63:
         pytest.skip("long double is binary64 here")
     normal_tables.write(str(tmp_path / "normal_tables.h"))
