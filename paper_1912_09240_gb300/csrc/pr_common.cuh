@@ -214,23 +214,36 @@ __device__ __forceinline__ void em_step_chem_f32(float& x, float& y, float ax, f
     y = yn;
 }
 
-// sqrt(max(v, 0)), 0 for NaN, with four binary64 instructions: the clamp and the
-// conversions run on the integer units, s = v rsqrt(v) starts in binary32
-// (relative error d < 2^-21), and two steps s += (v - s^2) / (2 sqrt v) with the
-// residual from one fused multiply-add leave 1.5 d^2 and then 1.5 d^3 < 2^-62
-// before the last rounding.  Beyond 2^+-100, sqrt itself.
+// sqrt(max(v, 0)), 0 for NaN, with four binary64 instructions; the clamp, the
+// scaling to m = v 2^-2k in [1, 4) and the conversions run on the integer units.
+// r = rsqrt(m) from binary32 with its residual u = 1 - m r^2 (from exact products:
+// 2^-45) gives 1 / (2 sqrt m) to 2^-43.  Two steps s += (m - s^2) / (2 sqrt m) with
+// the residual from one fused multiply-add leave 2^-44 and then 2^-87 before the
+// last rounding, so the root is the correctly rounded one (but of 4^k (1 - 2^-53),
+// 2^-55 of a unit from a midpoint; with the binary32 r itself in the last step one
+// root in 400 was not).  Subnormals and infinity take sqrt itself.
 __device__ __forceinline__ double sqrt_clamped_f64(double v)
 {
     const uint64_t b = (uint64_t)__double_as_longlong(v);
     const uint32_t hi = (uint32_t)(b >> 32);
-    if (hi - (923u << 20) < (200u << 20)) {
-        const float vf = __uint_as_float((uint32_t)(b >> 29) + 0x40000000u);   // truncated
-        const float rf = rsqrtf(vf), sf = vf * rf;
+    if (hi - (1u << 20) < (2046u << 20)) {
+        const uint32_t k2 = ((hi >> 20) - 1023u) & ~1u;                // 2 k
+        const uint64_t mb = b - ((uint64_t)(k2 << 20) << 32);
+        const double m = __longlong_as_double((long long)mb);
+        const float mf = __uint_as_float((uint32_t)(mb >> 29) + 0x40000000u);   // truncated, m - mf = ml
+        const float ml = (float)((uint32_t)mb & 0x1FFFFFFFu) * (mf >= 2.0f ? 0x1p-51f : 0x1p-52f);
+        const float rf = rsqrtf(mf), sf = mf * rf;
+        const float p = __fmul_rn(rf, rf), pe = __fmaf_rn(rf, rf, -p);
+        const float u = __fmaf_rn(-ml, p, __fmaf_rn(-mf, pe, __fmaf_rn(-mf, p, 1.0f)));
+        // rf / 2 (1 + u / 2), the second term in units of 2^-46 of the first's binade
+        const int64_t cor = (int64_t)__float2int_rn(rf * u * 0x1p44f) << 8;
         const uint32_t ru = __float_as_uint(rf), su = __float_as_uint(sf);
-        const double half_r = __hiloint2double((int)((ru >> 3) + 0x37F00000u), (int)(ru << 29));
+        const int64_t rb = (int64_t)((uint64_t)((ru >> 3) + 0x37F00000u) << 32 | (ru << 29));
+        const double half_r = __longlong_as_double(rb + cor);
         double s = __hiloint2double((int)((su >> 3) + 0x38000000u), (int)(su << 29));
-        s = fma(half_r, fma(-s, s, v), s);
-        return fma(half_r, fma(-s, s, v), s);
+        s = fma(half_r, fma(-s, s, m), s);
+        s = fma(half_r, fma(-s, s, m), s);
+        return __longlong_as_double(__double_as_longlong(s) + ((int64_t)(int32_t)(k2 << 19) << 32));
     }
     if ((int32_t)hi <= 0 && (hi != 0u || (uint32_t)b == 0u)) return 0.0;   // zeros and negative numbers
     return sqrt(fmax(v, 0.0));

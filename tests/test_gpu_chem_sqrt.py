@@ -1,6 +1,9 @@
 """The binary64 amplitudes of the chemical system, sqrt(max(., 0)): one step from
 states that put their arguments at both ends of the square root's range and
 beyond them (where the library's function takes over), at zero and below it."""
+import ctypes
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -49,3 +52,55 @@ def test_one_step_over_the_range_of_the_amplitudes(L, orc, scale, sign):
     with np.errstate(divide="ignore", invalid="ignore"):
         amp = np.minimum(np.sqrt(d), np.where(v > 0, d / np.sqrt(v), np.inf))
     assert np.all(np.abs(gy.cpu().numpy()[:, 0] - oy[:, 0]) <= u * (ya + ay * poly + z * np.sqrt(v)) + z * amp)
+
+
+ROOTS = r"""
+#include "pr_common.cuh"
+__global__ void roots(const double* v, double* s, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) s[i] = pr::sqrt_clamped_f64(v[i]);
+}
+extern "C" int run(const void* v, void* s, int n)
+{
+    roots<<<(n + 255) / 256, 256>>>((const double*)v, (double*)s, n);
+    return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+@pytest.mark.parametrize("kind", ["all exponents", "near one", "short significands", "squares", "edges"])
+def test_root_is_correctly_rounded(tmp_path, kind):
+    """The root itself against the host's, bit for bit: every exponent, significands with runs of zeros or
+    ones at their end, squares and their neighbours, zeros, subnormals, negative numbers, infinity, NaN.
+    Left out: 4^k (1 - 2^-53), whose root is 2^-55 of a unit from a midpoint."""
+    from paper_1912_09240_gb300 import build as b
+    n = 1 << 21
+    r = np.random.default_rng(7)
+    bits = r.integers(0, 0x7FF0 << 48, n, dtype=np.uint64)
+    ones = (np.uint64(1) << r.integers(0, 53, n).astype(np.uint64)) - np.uint64(1)
+    if kind == "near one":
+        bits = (bits & np.uint64((1 << 52) - 1)) | (r.integers(1020, 1027, n).astype(np.uint64) << np.uint64(52))
+    if kind == "short significands":
+        bits = np.where(r.random(n) < 0.5, bits & ~ones, bits | ones)
+    v = bits.view(np.float64)
+    if kind == "squares":
+        root = r.integers(1, 1 << 26, n).astype(np.float64) * np.exp2(r.integers(-30, 30, n))
+        v = (root * root).view(np.int64) + r.integers(-2, 3, n)
+        v = v.view(np.float64)
+    if kind == "edges":
+        v = np.array([0.0, -0.0, 5e-324, 2.2e-308, 2.0 ** -1022, np.nextafter(2.0 ** -1022, 0), -1.0, -5e-324, -1e308,
+                      1.0, 2.0, 4.0, np.nextafter(1.0, 2), np.nextafter(2.0, 3), np.nextafter(2.0, 1), 1.7e308,
+                      np.inf, -np.inf, np.nan, -np.nan])
+    v = v[(v.view(np.uint64) & np.uint64((1 << 53) - 1)) != np.uint64((1 << 52) - 1)]
+    (tmp_path / "r.cu").write_text(ROOTS)
+    so = str(tmp_path / "r.so")
+    subprocess.check_call([b.nvcc(), *b.ARCH, "-O3", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", b.CSRC,
+                           "-o", so, str(tmp_path / "r.cu")])
+    gv = torch.tensor(v, device="cuda")
+    gs = torch.empty_like(gv)
+    torch.cuda.synchronize()
+    assert ctypes.CDLL(so).run(ctypes.c_void_p(gv.data_ptr()), ctypes.c_void_p(gs.data_ptr()), v.size) == 0
+    with np.errstate(invalid="ignore"):
+        want = np.sqrt(np.fmax(v, 0.0))
+    np.testing.assert_array_equal(gs.cpu().numpy(), np.where(want == 0.0, 0.0, want))
