@@ -86,22 +86,27 @@ __device__ __forceinline__ float narrow(double v)
     return (float)v;
 }
 
-// a > b and a <= b on the integer units, false where either is a NaN (a binary64
-// comparison takes the FP64 pipe, 64 cycles of a sub-partition).
+// a > b on the integer units, false where either is a NaN (a binary64 comparison
+// takes the FP64 pipe, 64 cycles of a sub-partition).
 constexpr long long kKeyInf = 0x7FF0000000000000ll;
 __device__ __forceinline__ bool greater_f64(double a, double b)
 {
     const long long x = okey(a), y = okey(b);
     return x > y && x <= kKeyInf && y >= -kKeyInf;
 }
-__device__ __forceinline__ bool at_most_f64(double a, double b)
-{
-    const long long x = okey(a), y = okey(b);
-    return x <= y && x >= -kKeyInf && y <= kKeyInf;
-}
 
 // The larger of a (not a NaN) and b; a NaN in b is passed over.
-__device__ __forceinline__ double max_f64(double a, double b) { return greater_f64(b, a) ? b : a; }
+__device__ __forceinline__ double max_f64(double a, double b)
+{
+    const long long y = okey(b);
+    return y > okey(a) && y <= kKeyInf ? b : a;
+}
+
+// min(v, 1) for v >= 0; 1 for a NaN.
+__device__ __forceinline__ double at_most_one(double v)
+{
+    return (unsigned long long)__double_as_longlong(v) < 0x3FF0000000000000ull ? v : 1.0;
+}
 
 constexpr int kWsum = 56;   // doubles of the scratch `wsum` of the block-level helpers
 
@@ -288,7 +293,7 @@ __device__ inline void coarse_apply_block(const double* __restrict__ P, int I, c
     const int q0 = split ? d.lo(I - 1) : 0, q1 = split ? d.hi(I - 1) : I - 1;
     for (int r = q0 + threadIdx.x; r < q1; r += blockDim.x) {
         const double v = total > 0.0 ? __ddiv_rn(mp[r], total) : 0.0;
-        out[r + 1] = greater_f64(1.0, v) ? v : 1.0;
+        out[r + 1] = at_most_one(v);
     }
     if (threadIdx.x == 0) {
         out[0] = 0.0;
@@ -349,8 +354,11 @@ __device__ __forceinline__ void quantiles(const GridDev& g, const double* edges,
     const double t = __ddiv_rn(__dsub_rn(p, F[lt - 1]), __dsub_rn(F[lt], F[lt - 1]));
     const double e0 = edges[lt - 1], e1 = edges[lt];
     double q = __dadd_rn(e0, __dmul_rn(t, g.h));
-    if (at_most_f64(q, e0)) q = nextafter(e0, e1);
-    if (at_most_f64(e1, q)) q = nextafter(e1, e0);
+    const long long k = okey(q), k0 = okey(e0), k1 = okey(e1);
+    if (k <= k0 || k >= k1) {   // (a NaN stays one)
+        if (k <= k0 && k >= -kKeyInf) q = nextafter(e0, e1);
+        if (k >= k1 && k <= kKeyInf) q = nextafter(e1, e0);
+    }
     qm = qp = q;
 }
 
@@ -752,8 +760,10 @@ __device__ inline void quantile_iterate_block(const GridDev& g, int qmode, const
                 v = __dadd_rn(pj, __dmul_rn(t, __dsub_rn(pn, pj)));
             }
         }
-        if (greater_f64(0.0, v)) v = 0.0;   // (a NaN stays: the caller reports it)
-        if (greater_f64(v, 1.0)) v = 1.0;
+        if ((unsigned long long)__double_as_longlong(v) > 0x3FF0000000000000ull) {
+            if (greater_f64(0.0, v)) v = 0.0;   // (a NaN stays: the caller reports it)
+            if (greater_f64(v, 1.0)) v = 1.0;
+        }
         out[i] = v;
     }
     if (threadIdx.x == 0) {
