@@ -625,7 +625,10 @@ extern "C" pr_status pr_batch_create(const pr_problem* problems, int32_t n_probl
                          (int)coarse_apply_smem(pl->max_bins));
     cudaFuncSetAttribute(batch_restrict0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)((((size_t)(pl->max_bins + 1) * 4 + 15) & ~(size_t)15) + (size_t)pl->max_bins * 4));
-    pl->ppt = 2;   // 16 problems of 1e4..1e5 particles: an iteration 21.8 ms (four particles per thread 22.1 ms)
+    // until pr_batch_tune: an iteration of 64 problems of 1e4..1e6 particles 413 ms
+    // (four particles per thread 415, one 401), of 16 problems of 1e4..1e5 14.5 ms
+    // (14.8, 14.1), of 4 problems 15.4 ms (15.3, 14.8)
+    pl->ppt = 2;
     pl->item_work = 0.0;
     {
         const int slots = resident_ctas(*pl);

@@ -372,7 +372,7 @@ l2_density_kernel(GridDev g, const double* __restrict__ c1, const double* __rest
     if (threadIdx.x == 0) out[blockIdx.x] = sqrt(s);
 }
 
-// CTAs of the cluster that runs the serial sweep (1, 2, 4 or 8; portable sizes).
+// CTAs of the cluster that runs the serial sweep (1, 2, 4 or 8: the portable sizes; 16 not tried).
 static int g_update_cluster = 8;
 
 template <typename K>

@@ -364,14 +364,19 @@ __device__ __forceinline__ void quantiles(const GridDev& g, const double* edges,
 
 // Remote stores (Dist::share) go into mp, counted, kq and the CDFs `out` only.
 // Between an exchange's barrier and the next exchange the CTAs of a cluster run
-// apart, so the target of the next one must overlap nothing that a CTA still
-// uses in between (its own part of the target apart):
-//   mp       behind the barrier that ends the slice before (see serial_sweep)
-//   counted  behind share(mp); in between mass, mp, wsum and the CDFs
-//   kq       behind share(counted); in between counted, below, per, levels, bsum
-//            and the CDFs
-//   out      behind share(kq) (the coarse step's: share(mp)); in between none of
-//            its own kind
+// apart, so what the next one stores over must not be in use in between (its own
+// part apart).  Per target: the cluster barrier before the stores, and the last
+// use by another CTA that it follows:
+//   mp                  the read-back's exchange, or the barrier at the end of a
+//                       slice: the levels in the read-back, the division of mp
+//   out of the coarse   share(mp): the slice before (its CDF is copied or read
+//   step (above 256)    before the coarse step)
+//   counted             share(mp), and `out` above 256 bins: the repair of the slice
+//                       before; a CTA behind may still scan and divide mp
+//   kq                  share(counted): the read-back of the slice before; a CTA
+//                       behind may still merge into below, compact or take quantiles
+//   out of the          share(kq): its copy at the end of the slice before
+//   read-back
 struct JqSmem {
     double* levels;   // [3(I+1)]; before the iterator the coarse step's mass | mp [I] each
     double *mass, *mp;

@@ -34,8 +34,13 @@ constexpr int kMomThreads = 256;
 constexpr int kMomMaxOrder = 4;
 constexpr int kMomUnroll = 8;              // loads in flight per thread
 constexpr int64_t kMomPerBlock = 4096;     // particles per CTA at least (then fewer CTAs)
-constexpr int64_t kMomMaxBlocks = 1824;    // CTAs over all slices at most: 12 per SM of 152, two waves of the
-                                           // binary32 kernel's 6 (orders 1, 2), three of its 4 (orders 3, 4)
+// CTAs over all slices at most: 12 per SM of 152, two waves of the binary32
+// kernel's 6 (orders 1, 2), three of its 4 (orders 3, 4); a constant, so that a
+// call's bits do not depend on the device.  Against 16 per SM, 49 x 2^20 values:
+// binary32 45.5..154 us instead of 51..161 (orders 1..4), weighted 105..449 instead
+// of 110..454, binary64 115..565 instead of 118..566; the largest loss measured
+// 4 % (49.5 us instead of 47.5, 16 x 600,000 binary32 values, four orders).
+constexpr int64_t kMomMaxBlocks = 1824;
 
 static int64_t moments_blocks(int64_t n, int32_t n_slices)
 {

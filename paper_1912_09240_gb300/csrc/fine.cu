@@ -392,8 +392,8 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
 // Bound by the binary64 pipe (64 cycles of a sub-partition per warp
 // instruction): 8 operations per step of the double well, 6 of the OU family,
 // the pipe 85 % busy.  The normals come from integer arithmetic
-// (normal64.cuh), 232 of the 240 instructions of a step, beside them.  2^17
-// particles x 2 slices x 1000 steps of the double well: 4.71 ms (5.6e10
+// (normal64.cuh), 246 of the 254 instructions of a step, beside them.  2^17
+// particles x 2 slices x 1000 steps of the double well: 4.67 ms (5.6e10
 // particle-steps/s); 40.8 ms with log, sqrt and sincospi of the CUDA library,
 // which made 80 binary64 operations a step.
 // The normals' tables (92 KB) are copied into the CTA's shared memory where

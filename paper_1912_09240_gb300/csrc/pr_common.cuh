@@ -364,8 +364,7 @@ __device__ __forceinline__ double edge(const GridDev& g, int i)
     return __dadd_rn(g.lo, __dmul_rn(index_f64(i), g.h));
 }
 
-// Bin of a double: e_i <= x < e_{i+1}, clamped into [0, I-1].
-// The bin from binary32 arithmetic, or -1 where x is outside the grid, within the
+// The bin of a double from binary32 arithmetic, or -1 where x is outside the grid, within the
 // rounding errors of an edge (g.margin), or not a normal binary32 number.
 __device__ __forceinline__ int bin_try_f64(const GridDev& g, double x)
 {
@@ -379,6 +378,7 @@ __device__ __forceinline__ int bin_try_f64(const GridDev& g, double x)
     return f > g.margin && f < 1.0f - g.margin && (uint32_t)k < (uint32_t)g.bins ? k : -1;
 }
 
+// Bin of a double: e_i <= x < e_{i+1}, clamped into [0, I-1].
 __device__ __forceinline__ int bin_of_f64(const GridDev& g, double x)
 {
     const int k = bin_try_f64(g, x);
