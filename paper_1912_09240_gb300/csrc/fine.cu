@@ -213,7 +213,7 @@ fine_f32_d1_kernel(FineArgs a, FineSmemOffsets so, int flags)
 // (1+D) mod 4 from blocks shared by four consecutive steps.
 // ---------------------------------------------------------------------------
 
-template <int KIND, int D>
+template <int KIND, int D, bool SHARED>
 __global__ void __launch_bounds__(512)
 fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
 {
@@ -268,14 +268,16 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
     constexpr int FP = F > 0 ? 2 * F : 1;   // Box-Muller pairs of the full blocks
     constexpr int TP = T > 0 ? 2 * T : 1;   // pairs of a group's tail blocks
     const uint32_t k0 = a.k0, k1 = a.k1, chi = a.ctr_hi, pid = (uint32_t)p;
-    // The rounds' part that all particles share, for kSpan steps at a time: a
-    // lane makes block g of step m, the warp reads it back from shared memory.
+    // SHARED: the rounds' part that all particles share, for kSpan steps at a time: a
+    // lane makes block g of step m, the warp reads it back from shared memory.  Else
+    // whole blocks (small launches, see launch_f32_dn).
     constexpr int kSpan = F > 0 ? (F == 1 ? 32 : F == 2 ? 16 : 8) : 4;   // a multiple of 4, F kSpan <= 32
     uint4* shared_rounds = reinterpret_cast<uint4*>(smem + so.rounds) + 32 * (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const PhiloxParticle own = philox_particle(pid, slice, k0);
+    auto whole = [&](uint32_t c, uint32_t hi) { return philox4x32_10(make_uint4(c, pid, slice, hi), k0, k1); };
     auto fill_rounds = [&](int m) {
-        if (F > 0) {
+        if (SHARED && F > 0) {
             __syncwarp();
             if (lane < F * kSpan)
                 shared_rounds[lane] =
@@ -291,8 +293,10 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
     auto tail_blocks = [&](int m) {
 #pragma unroll
         for (int j = 0; j < T; ++j) {
-            const uint4 w = philox_finish(own, philox_shared((uint32_t)(m >> 2), slice, chi | (uint32_t)(F + j), k0, k1),
-                                          k0, k1);
+            uint4 w;
+            if constexpr (SHARED)
+                w = philox_finish(own, philox_shared((uint32_t)(m >> 2), slice, chi | (uint32_t)(F + j), k0, k1), k0, k1);
+            else w = whole((uint32_t)(m >> 2), chi | (uint32_t)(F + j));
             box_muller_qcs(w.x, w.y, tq[2 * j], tc[2 * j], ts[2 * j]);
             box_muller_qcs(w.z, w.w, tq[2 * j + 1], tc[2 * j + 1], ts[2 * j + 1]);
         }
@@ -303,14 +307,18 @@ fine_f32_dn_kernel(FineArgs a, FineSmemOffsets so, int flags)
     auto step = [&](int m, int s4) {
         float pq = 0.0f, pc = 0.0f, ps = 0.0f;   // Q = 2: this step's pair
         if (Q <= 2) {
-            const uint4 w = philox_finish(own, philox_shared((uint32_t)(m >> 1), slice, chi, k0, k1), k0, k1);
+            uint4 w;
+            if constexpr (SHARED) w = philox_finish(own, philox_shared((uint32_t)(m >> 1), slice, chi, k0, k1), k0, k1);
+            else w = whole((uint32_t)(m >> 1), chi);
             if (m & 1) box_muller_qcs(w.z, w.w, pq, pc, ps);
             else box_muller_qcs(w.x, w.y, pq, pc, ps);
         }
         float q[FP], c[FP], sn[FP], amp[FP];
 #pragma unroll
         for (int gi = 0; gi < F; ++gi) {
-            const uint4 w = philox_finish(own, shared_rounds[(m % kSpan) * F + gi], k0, k1);
+            uint4 w;
+            if constexpr (SHARED) w = philox_finish(own, shared_rounds[(m % kSpan) * F + gi], k0, k1);
+            else w = whole((uint32_t)m, chi | (uint32_t)gi);
             box_muller_qcs(w.x, w.y, q[2 * gi], c[2 * gi], sn[2 * gi]);
             box_muller_qcs(w.z, w.w, q[2 * gi + 1], c[2 * gi + 1], sn[2 * gi + 1]);
         }
@@ -864,7 +872,12 @@ static pr_status launch_f32_dn(const FineArgs& a, FineSmemOffsets so, int flags,
 {
     const int threads = fine_f32_threads(a.n, true);
     dim3 grid((unsigned)((a.n + threads - 1) / threads), (unsigned)n_slices);
-    auto k = fine_f32_dn_kernel<KIND, D>;
+    // Shared rounds save issue but add latency: they pay from three warps per
+    // sub-partition on.  1000 steps of d = 16, 8 and 4: 3000 particles (half a warp)
+    // 440, 246 and 174 us with them, 352, 195 and 141 without; 20,000 (four warps)
+    // 916, 504 and 306 us with, 948, 526 and 319 without.
+    const int64_t ctas_per_sm = ((int64_t)grid.x * n_slices + num_sms() - 1) / num_sms();
+    auto k = ctas_per_sm * threads > 2 * 128 ? fine_f32_dn_kernel<KIND, D, true> : fine_f32_dn_kernel<KIND, D, false>;
     PR_TRY_CUDA(set_smem(k, smem));
     k<<<grid, threads, smem, st>>>(a, so, flags);
     PR_CHECK_LAUNCH();

@@ -68,3 +68,29 @@ def test_adjoint_chunks_straddle_slices(L, n, slices, steps, ckpt):
                       seed, None, total, None, None, ws)
     want = (seed.cpu().numpy()[:, None] * DX[:, :3])
     assert np.all(np.abs(total.cpu().numpy() - want.sum(0)) <= TOL * np.abs(want).sum(0))
+
+
+@pytest.mark.parametrize("d", [2, 3, 4, 7, 8, 12, 14, 15, 16])
+@pytest.mark.parametrize("steps", [1, 3, 4, 6, 9, 34])
+def test_small_launches_take_whole_blocks(d, steps):
+    """The multi-component kernel draws whole blocks in launches of up to two warps per sub-partition and
+    shared rounds beyond: the first particles of a large ensemble end where they do in a small one."""
+    import torch
+    from paper_1912_09240_gb300 import _lib as L
+    from paper_1912_09240_gb300 import build as b
+    b.build()
+    n = 150_001                                   # two CTAs of 512 threads per SM
+    g = torch.Generator(device="cuda").manual_seed(d)
+    x = torch.randn(1, n, generator=g, device="cuda")
+    y = torch.randn(1, d, n, generator=g, device="cuda")
+    model = L.Model(L.PR_MODEL_DW_MULTI, d, 0.5, 1.0, 0.1)
+
+    def run(k):
+        xi, yi = (v[..., :k].clone(memory_format=torch.contiguous_format) for v in (x, y))   # (propagated in place)
+        L.pr_fine_propagate(model, L.PR_F32, L.Rng(9, 2), xi, yi, False, xi, yi, k, 4, 1, steps, 1e-3)
+        return xi, yi
+
+    full = run(n)
+    for k in (1, 63, 4097, 20_000):
+        part = run(k)
+        assert torch.equal(part[0], full[0][:, :k]) and torch.equal(part[1], full[1][:, :, :k])
