@@ -312,7 +312,8 @@ parareal_update_kernel(const double* __restrict__ P, GridDev g, int iterator, in
     serial_sweep<CL>(usm, P, g, iterator, qmode, K, cdf0, fstar, cstar, next, status);
 }
 
-__global__ void __launch_bounds__(kCoarseThreads, 1)
+template <int PER_SM>
+__global__ void __launch_bounds__(kCoarseThreads, PER_SM)
 iterate_kernel(GridDev g, int iterator, int qmode, const double* __restrict__ a, const double* __restrict__ b,
                const double* __restrict__ c, double* __restrict__ out, int32_t* status)
 {
@@ -626,10 +627,20 @@ extern "C" pr_status pr_iterate(pr_iterator iterator, pr_quantile_mode qmode, co
     if (status) PR_TRY_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
     const GridDev g = make_grid(*grid);
     const size_t smem = (size_t)4 * (grid->bins + 1) * sizeof(double) + jq_smem_bytes(grid->bins);
-    PR_TRY_CUDA(allow_smem(iterate_kernel, smem));
-    iterate_kernel<<<n_vec, kCoarseThreads, smem, st>>>(g, (int)iterator, (int)qmode, a, b, c, out, status);
-    PR_CHECK_LAUNCH();
-    return PR_OK;
+    auto launch = [&](auto kernel) -> pr_status {
+        PR_TRY_CUDA(allow_smem(kernel, smem));
+        kernel<<<n_vec, kCoarseThreads, smem, st>>>(g, (int)iterator, (int)qmode, a, b, c, out, status);
+        PR_CHECK_LAUNCH();
+        return PR_OK;
+    };
+    // as many CTAs per SM as the states and the shared memory make (registers cut
+    // for one, two or four): 400 states of 5 bins 17 us at four, 24 at two, 32 at
+    // one; of 512 bins 83 us at two, 105 at one, 88 with registers for four; of
+    // 1024 bins (one fits) 145 us, 150 with registers for two
+    const int64_t want = ((int64_t)n_vec + num_sms() - 1) / num_sms();
+    const int64_t per_sm = std::min<int64_t>(want, ((int64_t)smem_optin_max() + 1024) / (int64_t)(smem + 1024));
+    if (per_sm >= 3) return launch(iterate_kernel<4>);
+    return per_sm == 2 ? launch(iterate_kernel<2>) : launch(iterate_kernel<1>);
 }
 
 extern "C" pr_status pr_w1(const pr_grid* grid, int32_t n_vec, const double* c1, const double* c2, double* w1,

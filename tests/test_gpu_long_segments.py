@@ -63,3 +63,27 @@ def test_long_pooled_segments(name, bins, qmode):
     finally:
         L.pr_set_update_cluster(8)
         L.pr_coarse_destroy(h)
+
+
+@pytest.mark.parametrize("bins", [5, 64, 300, 512, 1024])
+@pytest.mark.parametrize("n", [1, 200, 500])
+def test_many_states_at_once(bins, n):
+    """One, two and more states per SM (and as few as the shared memory allows): each as if alone."""
+    import torch
+    from paper_1912_09240_gb300 import _lib as L
+    b.build()
+    names = sorted(CASES)
+    rows = [np.stack([np.asarray(CASES[names[k % len(names)]](bins)[f]) for k in range(n)]) for f in range(3)]
+    t = [torch.tensor(r, device="cuda") for r in rows]
+    for v in t:
+        v[:, -1] = 1.0
+    st = torch.empty(1, dtype=torch.int32, device="cuda")
+    for iterator in (0, 1, 3):
+        out = torch.empty_like(t[0])
+        L.pr_iterate(iterator, 0, L.Grid(bins, -3.0, 3.0), n, *t, out, st)
+        assert int(st.item()) == 0
+        for k in range(min(n, len(names))):
+            one = torch.empty(1, bins + 1, dtype=torch.float64, device="cuda")
+            L.pr_iterate(iterator, 0, L.Grid(bins, -3.0, 3.0), 1, *(v[k:k + 1].clone() for v in t), one, st)
+            same = out[k::len(names)]
+            assert torch.equal(same, one.expand_as(same))
